@@ -83,7 +83,10 @@ extern "C" {
 #define LBHPDE_MAX_DEG 31  /* highest degree of f^eq_j(phi) the kernels accept */
 #define LBHPDE_NU_TERMS 64 /* capacity of the generalised f^eq tables: (A + 1)(Dg + 1) <= 64 */
 
-#define LBHPDE_KERNEL_AUTO 0    /* the on-chip kernel (ONCHIP)                                 */
+#define LBHPDE_KERNEL_AUTO 0    /* the on-chip kernel (ONCHIP); a batch of one lattice and one    */
+                                /* kind of boundary that is too small to fill the GPU takes       */
+                                /* one-warp windows over many SMs (bit for bit the same results   */
+                                /* as ONCHIP, or STREAM on bounded grids, where those apply)      */
 #define LBHPDE_KERNEL_STREAM 1  /* one fused collide+stream launch per step through HBM        */
 #define LBHPDE_KERNEL_ONCHIP 2  /* instances that fit one CTA stay resident in registers for   */
                                 /* all steps; longer ones advance in temporally blocked        */

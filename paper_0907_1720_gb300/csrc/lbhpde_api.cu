@@ -79,6 +79,14 @@ struct Group {
     int *smembers = nullptr;
     std::vector<int2> sblocks_h;       // their node blocks (kChunk nodes each)
     int2 *sblocks = nullptr;
+    // the whole batch in one-warp windows (then the plans above are empty)
+    lbh::PackedWave wv_h;
+    lbk::WaveWin *wv_wins = nullptr;
+    unsigned char *wv_box = nullptr;
+    unsigned *wv_ctrl = nullptr;
+    int *wv_members = nullptr;  // bounded: the batch indices of the plan's members,
+    void *wv_ends = nullptr;    //   and f^eq(phi_b) of the steps of a launch,
+    int wv_steps = 0;           //   as many as this holds
 };
 
 }  // namespace
@@ -1013,6 +1021,58 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     return LBHPDE_OK;
 }
 
+// The one-warp windows (k_wave) hold a batch of one lattice and one kind of boundary that is small
+// enough to be bound by latency, unless a kernel was asked for.  Bounded FP32 D1Q5 members that
+// k_ring_nee holds stay there: it adds a node's flux differences in another order.
+int plan_waves(lbhpde_batch_s *bt, bool *taken) {
+    *taken = false;
+    Group *g = nullptr;
+    for (int gi = 0; gi < 4; ++gi) {
+        Group &q = gi < 2 ? bt->groups[gi] : bt->bgroups[gi - 2];
+        bt->dev_free(q.wv_wins);
+        bt->dev_free(q.wv_box);
+        bt->dev_free(q.wv_ctrl);
+        bt->dev_free(q.wv_members);
+        bt->dev_free(q.wv_ends);
+        q.wv_members = nullptr;
+        q.wv_ends = nullptr;
+        q.wv_wins = nullptr;
+        q.wv_box = nullptr;
+        q.wv_ctrl = nullptr;
+        q.wv_h = lbh::PackedWave{};
+        if (q.members.empty()) continue;
+        if (g) return LBHPDE_OK;
+        g = &q;
+    }
+    if (!g || bt->kernel != LBHPDE_KERNEL_AUTO || bt->K_req || bt->spl_req) return LBHPDE_OK;
+    const bool nee = bt->nbounded > 0;
+    std::vector<Seg> m;
+    for (int i : g->members) {
+        if (nee && lbh::ring_nee_ok(bt->esz, g->b, bt->segs_h[i])) return LBHPDE_OK;
+        m.push_back(bt->segs_h[i]);
+    }
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (!lbh::plan_wave(bt->esz, g->b, g->has_nu ? -1 : lbh::onchip_dc(g->b, g->maxD), nee, m, sms, g->wv_h)) {
+        g->wv_h = lbh::PackedWave{};
+        return LBHPDE_OK;
+    }
+    RC(bt->upload(&g->wv_wins, g->wv_h.wins));
+    RC(bt->dev_alloc((void **)&g->wv_box, g->wv_h.box_bytes));
+    RC(bt->dev_alloc((void **)&g->wv_ctrl, 4 * sizeof(unsigned)));
+    CK(cudaMemsetAsync(g->wv_box, 0, g->wv_h.box_bytes, bt->stream));
+    CK(cudaMemsetAsync(g->wv_ctrl, 0, 4 * sizeof(unsigned), bt->stream));
+    if (nee) {
+        const size_t per = bt->esz * (size_t)lbk::wave_end_elems(g->b, 1) * m.size();  // bytes a step
+        g->wv_steps = (int)std::min<size_t>(4096, std::max<size_t>(64, (size_t(4) << 20) / per));
+        RC(bt->upload(&g->wv_members, g->members));
+        RC(bt->dev_alloc(&g->wv_ends, per * g->wv_steps));
+    }
+    *taken = true;
+    return LBHPDE_OK;
+}
+
 int choose_kernels(lbhpde_batch_s *bt) {
     // captured streaming graphs hold the launches of the groups that streamed when they were
     // captured: a new plan may change that set, so they are rebuilt on the next long run
@@ -1022,6 +1082,9 @@ int choose_kernels(lbhpde_batch_s *bt) {
             if (gx) cudaGraphExecDestroy(gx);
         bt->graph[0] = bt->graph[1] = nullptr;
     }
+    bool taken = false;
+    RC(plan_waves(bt, &taken));
+    if (taken) return LBHPDE_OK;
     for (auto &g : bt->groups) {
         if (g.members.empty()) continue;
         g.onchip_ok = false;
@@ -1301,6 +1364,22 @@ int batch_step(lbhpde_batch_s *bt, long nsteps, const double *phib = nullptr, lo
     if (nsteps == 0) return LBHPDE_OK;
     const double *pbd = nullptr;
     if (bt->nbounded) RC(stage_boundary(bt, nsteps, phib, stride, on_device, &pbd));
+    for (int gi = 0; gi < 4; ++gi) {
+        Group &g = gi < 2 ? bt->groups[gi] : bt->bgroups[gi - 2];
+        if (g.wv_h.wins.empty()) continue;
+        for (long done = 0; done < nsteps;) {  // the whole batch, in place
+            const int n = (int)std::min<long>(nsteps - done, bt->nbounded ? g.wv_steps : 1L << 30);
+            if (bt->nbounded) {
+                RC(lbh::launch_wave_ends(g.wv_h, g.wv_ends, bt->segs, g.wv_members, bt->coefT, pbd, stride, done, n, bt->stream));
+                ++bt->launches;
+            }
+            RC(lbh::launch_wave(g.wv_h, g.wv_wins, g.wv_box, g.wv_ctrl, bt->st[bt->cur], bt->coefT, n, g.wv_ends, bt->stream));
+            ++bt->launches;
+            done += n;
+        }
+        bt->steps += nsteps;
+        return LBHPDE_OK;
+    }
     const int cur0 = bt->cur;
     bool any_periodic = false;
     for (auto &g : bt->groups)

@@ -12,6 +12,7 @@
 #include "lbhpde_kernels.cuh"
 #include "lbhpde_ring.cuh"
 #include "lbhpde_ring_nee.cuh"
+#include "lbhpde_wave.cuh"
 
 namespace lbh {
 
@@ -152,5 +153,29 @@ int pack_ring_nee(int b, int dc, const std::vector<NeeMember> &m, PackedNee &out
 int launch_ring_nee_f32(int dc, const PackedNee &p, const lbk::RingNeeInst *insts_d, const int *first_d,
                         const void *in, void *out, const void *coefT, const double *phib, long long stride,
                         long long step0, int nsteps, cudaStream_t st);
+
+// Small and medium grids in windows of one warp each (k_wave, lbhpde_wave.cu).
+struct PackedWave {
+    std::vector<lbk::WaveWin> wins;  // whole CTAs (and clusters): unused places have N = 0
+    int esz = 0, b = 0, dc = 0;
+    int K = 0, G = 0;  // positions a lane, lane groups a window's populations are split over
+    bool nee = false;
+    int tblk = 0;      // steps between two trades of the windows' borders
+    int csize = 0;     // CTAs of a cluster that holds whole instances; 0: boxes in global memory
+    int nmem = 0, nused = 0;  // members; windows that hold nodes
+    int wsmem = 0;     // shared-memory elements a window, beside the boxes
+    size_t smem = 0, box_bytes = 0;
+    int ncta() const { return (int)wins.size() / lbk::kWaveWarps; }
+};
+// Windows of the members (periodic, or bounded with Seg::pad = depth); false where some member does
+// not divide that way.
+bool pack_wave(const std::vector<lbk::Seg> &m, int b, int K, int G, int T, int csize, std::vector<lbk::WaveWin> &out);
+// The plan of a whole batch, where k_wave is the better kernel for it on a GPU of `sms` SMs.
+bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms, PackedWave &out);
+// nsteps steps, in place; ends: the table of launch_wave_ends for the same steps (bounded members).
+int launch_wave(const PackedWave &p, const lbk::WaveWin *wins, unsigned char *box, unsigned *ctrl, void *st, const void *coefT,
+                int nsteps, const void *ends, cudaStream_t stream);
+int launch_wave_ends(const PackedWave &p, void *ends, const lbk::Seg *segs, const int *members, const void *coefT,
+                     const double *phib, long long stride, long long step0, int nsteps, cudaStream_t st);
 
 }  // namespace lbh
