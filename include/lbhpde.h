@@ -83,10 +83,11 @@ extern "C" {
 #define LBHPDE_MAX_DEG 31  /* highest degree of f^eq_j(phi) the kernels accept */
 #define LBHPDE_NU_TERMS 64 /* capacity of the generalised f^eq tables: (A + 1)(Dg + 1) <= 64 */
 
-#define LBHPDE_KERNEL_AUTO 0    /* the on-chip kernel (ONCHIP); a batch of one lattice and one    */
-                                /* kind of boundary that is too small to fill the GPU takes       */
-                                /* one-warp windows over many SMs (bit for bit the same results   */
-                                /* as ONCHIP, or STREAM on bounded grids, where those apply)      */
+#define LBHPDE_KERNEL_AUTO 0    /* the fastest for the batch: the on-chip kernel (ONCHIP), or, with */
+                                /* the same results bit for bit as ONCHIP at 2 to 8 nodes a thread */
+                                /* or STREAM, one-warp windows over many SMs for a batch of one    */
+                                /* lattice and one kind of boundary too small to fill the GPU, and */
+                                /* one-warp strips for FP32 periodic members that fill it          */
 #define LBHPDE_KERNEL_STREAM 1  /* one fused collide+stream launch per step through HBM        */
 #define LBHPDE_KERNEL_ONCHIP 2  /* instances that fit one CTA stay resident in registers for   */
                                 /* all steps; longer ones advance in temporally blocked        */
@@ -223,8 +224,7 @@ int lbhpde_kernel_launches(lbhpde_t h, long long *count);
 /* Which kernel lbhpde_step uses (LBHPDE_KERNEL_*).  For the on-chip kernels: the nodes each
  * thread holds (FP32: 2, 4 or 8 on D1Q5, 4 or 8 on D1Q7; FP64: 2 or 4 on D1Q5, 4 on D1Q7; 16 on
  * FP32 D1Q5 polynomial models selects the 16-node resident kernel, which holds instances of up
- * to 8192 nodes and is the automatic choice there, longer ones taking windows of the default
- * size) and the steps per launch (resident instances: launch chunk; windows: steps per window, which
+ * to 8192 nodes, longer ones taking windows of the default size) and the steps per launch (resident instances: launch chunk; windows: steps per window, which
  * sets the halo to steps * max|e| nodes); 0 = automatic.  Returns LBHPDE_ERR_UNSUPPORTED for a
  * combination the library was not built with, leaving the previous choice in place. */
 int lbhpde_set_kernel(lbhpde_t h, int kernel, int nodes_per_thread, int steps_per_launch);
@@ -233,8 +233,8 @@ int lbhpde_set_kernel(lbhpde_t h, int kernel, int nodes_per_thread, int steps_pe
  * counterpart).  Times the compiled (nodes per thread, steps per window)
  * candidates for one precision, lattice (5 or 7) and f^eq degree on a synthetic periodic grid
  * of 2^22 (FP32) or 2^21 (FP64) nodes in temporally blocked windows, and keeps the fastest in a
- * process-wide table.  Batches and handles created afterwards use the tuned pair wherever
- * lbhpde_set_kernel did not fix one.  Outputs (each may be NULL): the chosen pair and its
+ * process-wide table.  Batches and handles created afterwards use the tuned pair in the windows of
+ * the on-chip kernel wherever lbhpde_set_kernel did not fix one.  Outputs (each may be NULL): the chosen pair and its
  * measured node-updates per second.  Allocates and frees about 235 MB of device memory on the
  * current device and synchronises. */
 int lbhpde_autotune(int precision, int lattice, int degree, int *nodes_per_thread, int *steps_per_launch,

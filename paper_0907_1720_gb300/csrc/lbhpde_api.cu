@@ -60,6 +60,11 @@ struct Group {
         int *cta_first = nullptr;
         int ncta() const { return host.ncta(); }
     } ring[lbh::kRingClasses], halo;  // resident instances by CTA size class; windows
+    // every member in strips of one warp each (then ring and halo are empty)
+    lbh::PackedStrip strip;
+    lbk::StripSeg *strip_segs = nullptr;
+    int *strip_first = nullptr;
+    bool windows() const { return halo.ncta() || strip.nwarps(); }  // advances through both buffers
     int K = 0, maxt = 0, tblk = 0;
     int Kr = 0;  // nodes per thread of the resident plans (lbh::kRingK: k_ring)
     int Kt = 0;  // nodes per thread of the tail of a plan in whole waves
@@ -817,9 +822,49 @@ int plan_onchip(lbhpde_batch_s *bt, Group &g, int K, int Kr, int tblk, bool forc
     return LBHPDE_OK;
 }
 
+void drop_strip(lbhpde_batch_s *bt, Group &g) {
+    bt->dev_free(g.strip_segs);
+    bt->dev_free(g.strip_first);
+    g.strip_segs = nullptr;
+    g.strip_first = nullptr;
+    g.strip = lbh::PackedStrip{};
+}
+
+// Every member of the group in strips (k_strip) through both buffers, if that is faster.
+int plan_strip(lbhpde_batch_s *bt, Group &g, int sms, bool *done) {
+    std::vector<Seg> m;
+    for (int i : g.members) m.push_back(bt->segs_h[i]);
+    const int dc = lbh::onchip_dc(g.b, g.maxD);
+    lbh::PackedStrip p;
+    if (sms > 0) lbh::pack_strip(g.b, m, p);
+    // (the estimate of the other kernels is up to a tenth low where a last wave is half filled:
+    // ensembles of 200 and 600 members)
+    *done = sms > 0 && lbh::strip_cost(g.b, p.nwarps(), sms) < 1.1 * lbh::cta_cost(bt->esz, g.b, dc, false, false, m, sms);
+    if (!*done) return LBHPDE_OK;
+    for (auto &pl : g.ring) {
+        bt->dev_free(pl.insts);
+        bt->dev_free(pl.cta_first);
+        pl = Group::Plan{};
+    }
+    bt->dev_free(g.halo.insts);
+    bt->dev_free(g.halo.cta_first);
+    g.halo = Group::Plan{};
+    g.waves = false;
+    g.strip = std::move(p);
+    RC(bt->upload(&g.strip_segs, g.strip.segs));
+    RC(bt->upload(&g.strip_first, g.strip.first));
+    g.tblk = lbk::strip_steps(g.b);
+    g.onchip_ok = true;
+    return LBHPDE_OK;
+}
+
 int launch_group(lbhpde_batch_s *bt, Group &g, bool halo, const void *in, void *out, int nsteps, cudaStream_t st,
                  int cls = lbh::kRingClasses - 1) {
     Group::Plan &pl = halo ? g.halo : g.ring[cls];
+    if (halo && g.strip.nwarps()) {
+        if (nsteps > 0) ++bt->launches;
+        return lbh::launch_strip(g.strip, g.strip_segs, g.strip_first, in, out, bt->coefT, nsteps, st);
+    }
     if (pl.ncta() > 0 && nsteps > 0) ++bt->launches;
     const int Kx = halo ? g.K : (g.waves && cls == 0 && g.Kt ? g.Kt : g.Kr);
     return lbh::launch_onchip(g.b, bt->esz, Kx, g.dc, halo, pl.host, pl.insts, pl.cta_first, in, out, bt->coefT,
@@ -1088,6 +1133,7 @@ int choose_kernels(lbhpde_batch_s *bt) {
     for (auto &g : bt->groups) {
         if (g.members.empty()) continue;
         g.onchip_ok = false;
+        drop_strip(bt, g);
         if (bt->kernel == LBHPDE_KERNEL_STREAM) continue;
         // K_req = kRingK asks for the 16-node resident kernel, whose windows keep the default (or
         // tuned) K; automatic choice: that kernel wherever it applies
@@ -1105,6 +1151,12 @@ int choose_kernels(lbhpde_batch_s *bt) {
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             (void)cudaGetLastError();
             sms = 0;
+        }
+        // strips wherever they are the faster kernel (lbh::strip_cost against lbh::cta_cost)
+        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0 && lbh::strip_ok(bt->esz, g.b, dcg)) {
+            bool done = false;
+            RC(plan_strip(bt, g, sms, &done));
+            if (done) continue;
         }
         const bool small = bt->K_req == 0 && bt->kernel != LBHPDE_KERNEL_HALO && thr16 < 32LL * sms;
         int K_small = 0;
@@ -1143,7 +1195,7 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps) {
     for (auto &g : bt->groups) {
         if (g.members.empty()) continue;
         if (!g.onchip_ok) any_stream = true;
-        else if (g.halo.ncta()) any_halo = true;
+        else if (g.windows()) any_halo = true;
     }
     if (any_stream) {
         // one fused collide+stream launch per step, ping-pong buffers
@@ -1201,8 +1253,14 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps) {
     // read the current buffer once and write the buffer the halo launches end in
     int tb = 1 << 30;
     for (auto &g : bt->groups)
-        if (!g.members.empty() && g.halo.ncta()) tb = std::min(tb, g.tblk);
-    const long nchunks = any_halo ? (nsteps + tb - 1) / tb : 0;
+        if (!g.members.empty() && g.windows()) tb = std::min(tb, g.tblk);
+    long nchunks = any_halo ? (nsteps + tb - 1) / tb : 0;
+    // a captured call is replayed with the buffers it was captured with: it has to end in the one it
+    // began in (an even number of launches, or a copy back after a single step)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool captured = (nchunks & 1) && bt->stream != nullptr && cudaStreamIsCapturing(bt->stream, &cap) == cudaSuccess &&
+                          cap != cudaStreamCaptureStatusNone;
+    if (captured && nsteps > 1) ++nchunks;
     const int cur0 = bt->cur, cur1 = bt->cur ^ (int)(nchunks & 1);
     // resident instances (each size class) and windows touch disjoint rows: when there is more
     // than one kind, they run concurrently, the resident classes on streams of their own
@@ -1251,9 +1309,9 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps) {
     }
     long left = nsteps;
     for (long c = 0; c < nchunks; ++c) {
-        const int n = (int)std::min<long>(left, tb);
+        const int n = (int)((left + nchunks - c - 1) / (nchunks - c));  // equal parts, at most tb
         for (auto &g : bt->groups)
-            if (!g.members.empty() && g.halo.ncta())
+            if (!g.members.empty() && g.windows())
                 RC(launch_group(bt, g, true, bt->st[bt->cur], bt->st[bt->cur ^ 1], n, bt->stream));
         bt->cur ^= 1;
         left -= n;
@@ -1262,6 +1320,10 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps) {
         for (int c = 0; c < lbh::kRingClasses; ++c)
             if (used[c]) CK(cudaStreamWaitEvent(bt->stream, bt->ev_join[c], 0));
     bt->cur = cur1;
+    if (captured && cur1 != cur0) {
+        CK(cudaMemcpyAsync(bt->st[cur0], bt->st[cur1], bt->st_bytes, cudaMemcpyDeviceToDevice, bt->stream));
+        bt->cur = cur0;
+    }
     return LBHPDE_OK;
 }
 

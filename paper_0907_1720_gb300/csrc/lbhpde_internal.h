@@ -12,6 +12,7 @@
 #include "lbhpde_kernels.cuh"
 #include "lbhpde_ring.cuh"
 #include "lbhpde_ring_nee.cuh"
+#include "lbhpde_strip.cuh"
 #include "lbhpde_wave.cuh"
 
 namespace lbh {
@@ -177,5 +178,25 @@ int launch_wave(const PackedWave &p, const lbk::WaveWin *wins, unsigned char *bo
                 int nsteps, const void *ends, cudaStream_t stream);
 int launch_wave_ends(const PackedWave &p, void *ends, const lbk::Seg *segs, const int *members, const void *coefT,
                      const double *phib, long long stride, long long step0, int nsteps, cudaStream_t st);
+
+// Strips of one warp each (k_strip, lbhpde_strip.cu): warp w < nmix() holds segs[first[w] .. first[w + 1]),
+// warp nmix() + i holds segs[i] alone (i < nfull).
+struct PackedStrip {
+    std::vector<lbk::StripSeg> segs;
+    std::vector<int> first;
+    int b = 0, nfull = 0;
+    int nmix() const { return first.empty() ? 0 : (int)first.size() - 1; }
+    int nwarps() const { return nfull + nmix(); }
+};
+// Whether members of (element size, lattice, on-chip degree code) can take k_strip.
+bool strip_ok(size_t esz, int b, int dc);
+void pack_strip(int b, const std::vector<lbk::Seg> &m, PackedStrip &out);
+// What a step costs on a GPU of `sms` SMs, in SM clocks: the CTA-wide kernels on a group's members,
+// k_strip with that many warps.
+double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms);
+double strip_cost(int b, int nwarps, int sms);
+// At most lbk::strip_steps(b) steps, from buffer `in` to another one.
+int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
+                 const void *coefT, int nsteps, cudaStream_t st);
 
 }  // namespace lbh

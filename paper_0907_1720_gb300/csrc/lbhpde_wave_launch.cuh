@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "lbhpde.h"
 #include "lbhpde_internal.h"
@@ -245,33 +246,62 @@ long long wave_windows(const lbk::Seg &s, int W, int cap, int T) {
     return nee ? 2 + std::max<long long>(0, ((long long)s.N - 2 * (cap - H) + vin - 1) / vin) : ((long long)s.N + vin - 1) / vin;
 }
 
-// The step of the other kernels on the same members, in the same clocks: the CTA with the most nodes
-// (its barrier and exchange, then its nodes at the rate of one SM), or all nodes at the rate of the
-// GPU.  Measured at both ends: KdV on 400 nodes 580 (FP32) and 8080 (FP64) clocks, 2048-node FP64
-// windows 36 200, 1024-node FP32 windows 890, 2048-node D1Q7 ones 1930; bounded, 601 nodes: FP64
-// 16 400 (D1Q5) and 29 800 (D1Q7), FP32 D1Q7 2400; streamed (two launches a step): FP64 55 000 and
-// 84 900, FP32 23 400 and 29 700.
-double other_cost(size_t esz, int b, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms, double ops) {
-    const double rate = esz == 8 ? 2.0 / 1.08 : 128.0 / 1.35;  // FP operations a clock of an SM
-    const int cap = esz == 8 ? (b == 5 ? 2048 : 1024) : (b == 5 ? 1024 : 2048);
-    double worst = 0, total = 0;
+}  // namespace
+
+// The step of the CTA-wide kernels on a group's members, in SM clocks (GB300; measured in brackets).
+//   A CTA alone: a barrier and an exchange, then its nodes at the rate of one SM (KdV on 400 nodes
+//   [580 FP32, 8080 FP64], 2048-node FP64 windows [36 200]).
+//   FP32 windows: D1Q5 900 and then 5.2e11 node-updates/s [600 000 nodes 2430, 2^21 6390], D1Q7 1840 a
+//   wave of 152 windows [400 000 nodes 3620, 10^6 7060].
+//   FP32 D1Q5 residents of a group that fills the GPU (k_ring): 3400 a wave of 152 CTAs of 8192 nodes
+//   [ensemble of 128 members 3430, 400 6730, 4096 47 500].
+//   Bounded: 601 nodes FP64 [16 400 D1Q5, 29 800 D1Q7], FP32 D1Q7 [2400]; streamed, two launches a
+//   step: FP64 [55 000, 84 900], FP32 [23 400, 29 700].
+double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms) {
+    int D = 0;
+    long long total = 0;
     for (const lbk::Seg &s : m) {
+        D = std::max(D, s.D);
         total += s.N;
+    }
+    const double ops = wave_ops(b, dc > 0 ? dc : D), rate = esz == 8 ? 2.0 / 1.08 : 128.0 / 1.35;
+    const bool q5 = esz == 4 && b == 5, ring = q5 && dc >= 0 && !nee && total >= 32LL * kRingK * sms;
+    const int cap = esz == 8 ? (b == 5 ? 2048 : 1024) : (ring ? 512 * kRingK : (b == 5 ? 4096 : 2048));
+    const int window = q5 ? 1024 : cap;
+    double worst = 0, resident = 0, windows = 0;
+    for (const lbk::Seg &s : m) {
         double t;
         if (nee && s.N > kBoundedK * kBoundedMaxT)
             t = esz == 8 ? (b == 5 ? 55000 : 84900) : (b == 5 ? 23400 : 29700);
         else if (nee)
             t = s.N * ops / rate + (esz == 8 ? (b == 5 ? 5600 : 10000) : 1500);
         else if (real && esz == 8)
-            t = 94000;  // streamed (measured 45 us a step at 100 nodes, 65 at 1000 to 50 000)
+            t = 94000;  // streamed [45 us a step at 100 nodes, 65 at 1000 to 50 000]
         else
-            t = std::min(s.N, cap) * ops / rate + (esz == 8 ? 1500 : 520) + (real ? 1200 : 0);
+            t = (s.N <= cap ? s.N : window) * ops / rate + (esz == 8 ? 1500 : 520) + (real ? 1200 : 0);
+        (s.N <= cap || nee ? resident : windows) += s.N;
         worst = std::max(worst, t);
     }
-    return std::max(worst, total * ops / (rate * sms));
+    double all = (resident + windows) * ops / (rate * sms);
+    if (esz == 4 && !nee) {
+        const double waves = resident / (512.0 * kRingK * sms), rest = waves - (long long)waves;
+        const double res = ring ? 3400 * ((long long)waves + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0))) : resident * ops / (60.0 * sms);
+        const double win = windows == 0 ? 0 : (b == 5 ? 450 + windows * ops / (66.0 * sms) : 1840 * std::ceil(windows / (1856.0 * sms)) * ops / wave_ops(7, 7));
+        all = res + win;
+    }
+    return std::max(worst, all);
 }
 
-}  // namespace
+// A step of k_strip: one warp on a scheduler, two, and every further wave of two (GB300: D1Q5 400 000
+// nodes 2160, 800 000 3440, 2^24 37 800; D1Q7 400 000 2840, 800 000 4800, 2^24 75 400).
+double strip_cost(int b, int nwarps, int sms) {
+    const double one = b == 5 ? 2100 : 2840, two = b == 5 ? 3440 : 4800, more = b == 5 ? 2570 : 3620;
+    const double waves = nwarps / (8.0 * sms);
+    if (waves <= 0.5) return one;
+    if (waves <= 1.0) return two;
+    const double full = std::floor(waves), rest = waves - full;
+    return two + (full - 1) * more + (rest == 0 ? 0.0 : (rest <= 0.5 ? 0.54 * more : more));
+}
 
 bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms, PackedWave &out) {
     out = PackedWave{};
@@ -318,7 +348,12 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
             }
     }
     std::stable_sort(picks.begin(), picks.end(), [](const WavePick &x, const WavePick &y) { return x.cost < y.cost; });
-    const double other = other_cost(esz, b, nee, real, m, sms, ops);
+    double other = cta_cost(esz, b, dc, nee, real, m, sms);
+    if (!nee && strip_ok(esz, b, dc)) {
+        PackedStrip p;
+        pack_strip(b, m, p);
+        other = std::min(other, strip_cost(b, p.nwarps(), sms));
+    }
     for (const WavePick &k : picks) {
         if (k.cost > 0.85 * other) return false;
         out.esz = (int)esz;

@@ -1,0 +1,92 @@
+"""The FP32 strips (the automatic choice for periodic members that fill the GPU) against the streaming
+kernel: the update of a node is the same sequence of operations, so every result is equal (the
+streaming kernel itself is held to the oracle by the parity tests).  Sizes sit at the edges: the
+smallest grids, lengths that are not multiples of four, one node more or less than a strip owns
+(960 on D1Q5, 672 on D1Q7) and than its lanes hold; step counts below, at and above what one launch
+takes (16); one-step calls; a captured call that is replayed."""
+import numpy as np
+import pytest
+
+from paper_0907_1720_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0907_1720_gb300 import build as B
+    B.build()
+    from paper_0907_1720_gb300 import lbhpde
+    lbhpde.lib()
+    return lbhpde
+
+
+EQS = {"kdv": (lambda i: W.kdv_burgers(1.0 + 0.2 * i % 5, 0.01 * (i % 9), 0.5 + 0.01 * (i % 50)), 1e-4, 1.15),
+       "kawahara": (lambda i: W.kawahara(1.0, 0.5 + 0.01 * (i % 50), -1.0), 1e-4, 2.02)}
+
+
+def members(eq, sizes):
+    make, dt, tau = EQS[eq]
+    out = []
+    for i, N in enumerate(sizes):
+        rng = np.random.default_rng([N, i])
+        phi0 = 0.4 + 0.3 * np.cos(2 * np.pi * (np.arange(N) / N + rng.random())) + 0.01 * rng.standard_normal(N)
+        out.append(W.Problem(make(i), int(N), 0.1, dt, tau, 0, phi0))
+    return out
+
+
+def sizes(own, K):
+    edge = [6, 7, 31, K - 1, K, K + 1, own - 1, own, own + 1, own + K + 3, 2 * own, 2 * own + 5, 4099]
+    return edge + list(np.random.default_rng(own).integers(256, 8193, 700))
+
+
+def solve(L, ps, kernel, calls):
+    b = L.Batch(ps, precision=L.FP32_DEV).set_kernel(kernel)
+    b.set_phi(np.concatenate([p.phi0 for p in ps]))
+    launches = []
+    for n in calls:
+        n0 = b.kernel_launches()
+        b.step(n)
+        launches.append(b.kernel_launches() - n0)
+    out = b.read_phi()
+    b.close()
+    return out, launches
+
+
+@pytest.mark.parametrize("eq,own,K", [("kdv", 960, 32), ("kawahara", 672, 24)])
+def test_batch(L, eq, own, K):
+    ps = members(eq, sizes(own, K))
+    a, n = solve(L, ps, L.KERNEL_AUTO, [1, 15, 16, 17, 33])
+    b, _ = solve(L, ps, L.KERNEL_STREAM, [82])
+    assert n == [1, 1, 1, 2, 3]  # launches of at most 16 steps
+    assert np.isfinite(b).all() and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("eq,N", [("kdv", (1 << 22) + 3), ("kawahara", (1 << 21) + 1)])
+def test_long_grid(L, eq, N):
+    ps = members(eq, [N])
+    a, n = solve(L, ps, L.KERNEL_AUTO, [40])
+    b, _ = solve(L, ps, L.KERNEL_STREAM, [40])
+    assert n == [3] and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("steps", [1, 16, 40])
+def test_replayed_capture(L, steps):
+    ps = members("kdv", sizes(960, 32))
+    want, _ = solve(L, ps, L.KERNEL_STREAM, [3 * steps])
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        b = L.Batch(ps, precision=L.FP32_DEV)
+        b.set_phi(np.concatenate([p.phi0 for p in ps]))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            b.step(steps)
+        for _ in range(3):
+            g.replay()
+        got = b.read_phi()
+        b.close()
+    assert np.array_equal(got, want)
