@@ -463,17 +463,73 @@ int pack_ring(int b, size_t esz, int K, int dc, const std::vector<Member> &m, Pa
     return LBHPDE_OK;
 }
 
-int pack_halo(int b, size_t esz, int K, int dc, int H, const std::vector<Member> &m, Packed &out, bool wide) {
+// FP64 windows.  A multiply-add holds a scheduler's FP64 lanes for 64 clocks, so a step costs an SM the
+// warps it holds, whatever does the work, and what can be saved is copies, half-empty warps and SMs
+// that wait for the last ones.  A window is a CTA of P positions, a multiple of a warp's 128; an SM takes
+// ceil(n / SMs) of the n windows; a launch of T steps (copies T max|e| on either side) costs 8.5 us and
+// 0.6 us per 1000 positions of an SM on top.  With these, measured and (predicted) on GB300, us a
+// step: Kawahara on 2000003 nodes, P = 896 and T = 2: 214 (214), P = 768 and T = 4: 216 (216), against 237
+// for P = 1024 and T = 16; 300001 nodes: 33.0 (33) against 47.8; the ensemble of 256 members, P = 384 and
+// T = 4: 70.4 (70.9) against 82.7 with members up to 2048 nodes resident.
+bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps) {
+    const int W = lbk::wmax(b), most = std::min(onchip_maxt_halo(8, b, K), 256) * K, cap = onchip_maxt(8, b, K) * K;
+    int D = dc > 0 ? dc : 0;
+    long long resident = 0, windows = 0, large = 0;
+    for (const lbk::Seg &s : m) {
+        D = std::max(D, s.D);
+        if (s.N <= cap) {
+            resident += s.N;
+            large += s.N > cap / 2;
+        }
+    }
+    const double us = ((b - 1) * (D + 3) + 1) / 2.0 * 1.039 / 2070.0;  // of one position on an SM
+    const double multi = m.size() > 1 ? 0.25 : 0.0;
+    auto cost = [&](long long n, int P, int T) {
+        const double pos = (double)((n + sms - 1) / sms) * P;
+        return (pos + multi * P) * us + (T > 0 ? (8.5 + 0.0006 * pos) / T : 0.0);
+    };
+    // the plan without this choice: residents in CTAs of `cap` positions, windows of the default depth
+    const int T0 = default_tblk(cap, W);
+    for (const lbk::Seg &s : m)
+        if (s.N > cap) windows += (s.N + cap - 2 * T0 * W - 1) / (cap - 2 * T0 * W);
+    const long long nres = std::max((resident + cap - 1) / cap, large);
+    double best = cost(windows + nres, cap, windows ? T0 : 0);
+    *threads = 0;
+    for (int P = 256; P <= most; P += 32 * K)
+        for (int T : {2, 3, 4, 6, 8, 12, 16}) {
+            const int v = P - 2 * T * W;
+            if (v < P / 2) break;
+            long long n = 0;
+            for (const lbk::Seg &s : m) n += (s.N + v - 1) / v;
+            const double c = cost(n, P, T);
+            if (c < 0.97 * best) {
+                best = c;
+                *threads = P / K;
+                *steps = T;
+            }
+        }
+    return *threads > 0;
+}
+
+int pack_halo(int b, size_t esz, int K, int dc, int H, const std::vector<Member> &m, Packed &out, bool wide, int threads) {
     out = Packed{};
-    const int maxt = wide ? onchip_maxt(esz, b, K) : onchip_maxt_halo(esz, b, K);
+    int maxt = wide ? onchip_maxt(esz, b, K) : onchip_maxt_halo(esz, b, K);
     if (maxt == 0) return LBHPDE_ERR_UNSUPPORTED;
+    if (threads > 0) maxt = std::min(maxt, threads);
     const int valid = maxt * K - 2 * H;
     if (valid < 32) return LBHPDE_ERR_UNSUPPORTED;
     size_t coef_max = 0;
     for (const Member &mb : m) {
         const Seg &s = mb.seg;
-        for (long long x = 0; x < s.N; x += valid) {
-            const int v = (int)std::min<long long>(valid, s.N - x);
+        // windows of at most `valid` nodes; with a CTA size asked for, equal ones (a multiple of K
+        // nodes each, so that all but the last keep their vector loads)
+        long long part = valid;
+        if (threads > 0) {
+            const long long nw = (s.N + valid - 1) / valid;
+            part = std::min<long long>(valid, ((s.N + nw - 1) / nw + K - 1) / K * K);
+        }
+        for (long long x = 0; x < s.N; x += part) {
+            const int v = (int)std::min<long long>(part, s.N - x);
             OnchipInst I{};
             I.off = s.off;
             I.off2 = mb.off2;
@@ -750,7 +806,8 @@ int upload_plan(lbhpde_batch_s *bt, Group::Plan &pl) {
 // Nodes a thread of the tail of a plan in whole waves (members that fit it; the others keep 16)
 constexpr int kTailK = 8;
 
-int plan_onchip(lbhpde_batch_s *bt, Group &g, int K, int Kr, int tblk, bool force_halo) {
+// wthr: threads of a window CTA (0: the configuration's), each member then cut into equal windows.
+int plan_onchip(lbhpde_batch_s *bt, Group &g, int K, int Kr, int tblk, bool force_halo, int wthr = 0) {
     g.onchip_ok = false;
     const int maxt = lbh::onchip_maxt(bt->esz, g.b, Kr);
     if (maxt == 0 || K < lbk::wmax(g.b) || lbh::onchip_maxt(bt->esz, g.b, K) == 0) return LBHPDE_ERR_UNSUPPORTED;
@@ -812,7 +869,7 @@ int plan_onchip(lbhpde_batch_s *bt, Group &g, int K, int Kr, int tblk, bool forc
         RC(lbh::pack_ring(g.b, bt->esz, Kc, g.dc, ring[c], g.ring[c].host, threads));
         RC(upload_plan(bt, g.ring[c]));
     }
-    if (!halo.empty()) RC(lbh::pack_halo(g.b, bt->esz, K, g.dc, H, halo, g.halo.host));
+    if (!halo.empty()) RC(lbh::pack_halo(g.b, bt->esz, K, g.dc, H, halo, g.halo.host, false, wthr));
     RC(upload_plan(bt, g.halo));
     g.K = K;
     g.Kr = Kr;
@@ -1181,7 +1238,19 @@ int choose_kernels(lbhpde_batch_s *bt) {
         // FP64 real exponents: the FP64 pow binds both kernels, and streaming was faster on GB300
         // (3.88e9 node-updates/s against 3.62e9 in windows on a 2^24-node gKdV grid)
         if (g.has_nu && bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO) continue;
-        int rc = plan_onchip(bt, g, K, ring16 ? lbh::kRingK : K, tblk, bt->kernel == LBHPDE_KERNEL_HALO);
+        // FP64: windows of the size and depth that load the SMs evenly, for members of any length
+        // where that beats keeping the short ones resident
+        int wthr = 0, wsteps = 0;
+        if (bt->esz == 8 && !g.has_nu && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0 && tk == 0 && sms > 0) {
+            std::vector<Seg> m;
+            for (int i : g.members) m.push_back(bt->segs_h[i]);
+            const int Kd = lbh::default_K(bt->esz, g.b);
+            if (lbh::windows_f64(g.b, dcg, Kd, m, sms, &wthr, &wsteps)) {
+                K = Kd;
+                tblk = wsteps;
+            }
+        }
+        int rc = plan_onchip(bt, g, K, ring16 ? lbh::kRingK : K, tblk, bt->kernel == LBHPDE_KERNEL_HALO || wthr > 0, wthr);
         if (rc != LBHPDE_OK) return rc;
     }
     for (auto &g : bt->bgroups)

@@ -93,8 +93,12 @@ void split_ring_classes(size_t esz, int b, int K, const std::vector<Member> &m, 
 // Temporally blocked windows with halo H: one window per CTA.
 // wide: windows as large as a resident CTA (fewer, longer windows: the server, whose step
 // blocks fix the steps per window) instead of the smaller window CTAs.
+// threads > 0: windows of CTAs of at most that many threads, each member cut into equal ones.
 int pack_halo(int b, size_t esz, int K, int dc, int H, const std::vector<Member> &m, Packed &out,
-              bool wide = false);
+              bool wide = false, int threads = 0);
+// Whether FP64 periodic members advance faster in windows of a chosen size alone (threads of a CTA,
+// steps a launch) than with the short ones resident and the long ones in windows of the default size.
+bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps);
 
 // K == kRingK launches k_ring (resident plans only).
 int launch_onchip(int b, size_t esz, int K, int dc, bool halo, const Packed &p, const lbk::OnchipInst *insts_d,

@@ -1,4 +1,4 @@
-"""The FP32 strips (the automatic choice for periodic members that fill the GPU) against the streaming
+"""The FP32 strips and the FP64 windows (the automatic choices for periodic members that fill the GPU) against the streaming
 kernel: the update of a node is the same sequence of operations, so every result is equal (the
 streaming kernel itself is held to the oracle by the parity tests).  Sizes sit at the edges: the
 smallest grids, lengths that are not multiples of four, one node more or less than a strip owns
@@ -90,3 +90,19 @@ def test_replayed_capture(L, steps):
         got = b.read_phi()
         b.close()
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("eq,sizes64", [("kdv", [200003]), ("kawahara", [150001]), ("kdv", [6, 255, 257, 640, 2048, 2049, 8191] * 16),
+                                        ("kawahara", [7, 1000, 1025, 3001] * 24)])
+def test_fp64_windows(L, eq, sizes64):
+    """FP64 members in windows of a chosen size (equal parts of every member) against the streaming
+    kernel, equal; step counts that end in either buffer."""
+    ps = members(eq, sizes64)
+    phi0 = np.concatenate([p.phi0 for p in ps])
+    out = []
+    for kernel in (L.KERNEL_AUTO, L.KERNEL_STREAM):
+        b = L.Batch(ps, precision=L.FP64).set_kernel(kernel)
+        b.set_phi(phi0).step(1).step(16).step(25)
+        out.append(b.read_phi())
+        b.close()
+    assert np.isfinite(out[1]).all() and np.array_equal(out[0], out[1])
