@@ -75,7 +75,7 @@ struct Group {
     // bounded groups (LBHPDE_NEE): resident members, one CTA each, and streaming members
     std::vector<lbk::BoundedInst> bnd_h;
     lbk::BoundedInst *bnd = nullptr;
-    int bnd_threads = 0, bnd_dc = 0, bnd_D = 0;
+    int bnd_threads = 0, bnd_dc = 0, bnd_D = 0, bnd_K = 0;
     lbh::PackedNee rn_h;               // bounded members on the 16-node resident kernel
     lbk::RingNeeInst *rn_insts = nullptr;
     int *rn_first = nullptr;
@@ -1055,14 +1055,25 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.bnd_h.clear();
     g.smembers_h.clear();
     g.sblocks_h.clear();
-    const int K = lbh::kBoundedK;
+    int K = lbh::kBoundedK;
+    const int K4 = K;
+    if (bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && !g.has_nu && lbh::onchip_dc(g.b, g.maxD) > 0) {
+        std::vector<Seg> m;
+        for (int i : g.members)
+            if (bt->N[i] <= (long long)K * lbh::kBoundedMaxT) m.push_back(bt->segs_h[i]);
+        int dev = 0, sms = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (!m.empty() && sms > 0) K = lbh::bounded_nodes(g.b, m, sms);
+    }
+    g.bnd_K = K;
     int maxthr = 0, maxD = 0, maxDn = 0;
     bool real = false;
     // FP32 D1Q5 polynomial members take the 16-node resident kernel (unless a kernel or 4 nodes
     // a thread was asked for), the others one CTA each (real-exponent members on its variant
     // with the generalised f^eq) or the streaming step
     std::vector<lbh::NeeMember> nee;
-    const bool nee_auto = bt->kernel == LBHPDE_KERNEL_AUTO || (bt->kernel == LBHPDE_KERNEL_ONCHIP && bt->K_req != K);
+    const bool nee_auto = bt->kernel == LBHPDE_KERNEL_AUTO || (bt->kernel == LBHPDE_KERNEL_ONCHIP && bt->K_req != K4);
     for (int i : g.members) {
         const Seg &sg = bt->segs_h[i];
         if (nee_auto && lbh::ring_nee_ok(bt->esz, g.b, sg)) {
@@ -1071,7 +1082,7 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
             continue;
         }
         const int shift =
-            bt->N[i] <= (long long)K * lbh::kBoundedMaxT ? lbh::bounded_shift(g.b, sg.N, sg.pad) : -1;
+            bt->N[i] <= (long long)K4 * lbh::kBoundedMaxT ? lbh::bounded_shift(g.b, sg.N, sg.pad, K) : -1;
         if (bt->kernel != LBHPDE_KERNEL_STREAM && shift >= 0) {
             lbk::BoundedInst I{};
             I.off = sg.off;
@@ -1467,7 +1478,7 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
                 const size_t smem = lbh::bounded_smem(g.b, bt->esz, g.bnd_threads, g.bnd_D, n);
                 RC(lbh::launch_bounded(g.b, bt->esz, g.bnd_dc, (int)g.bnd_h.size(), g.bnd_threads, smem, g.bnd,
                                        bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT, pbd, stride,
-                                       done, n, bt->stream));
+                                       done, n, bt->stream, g.bnd_K));
                 ++bt->launches;
                 done += n;
             }

@@ -118,6 +118,7 @@ int launch_init(int b, size_t esz, void *st, const lbk::Seg *segs, const int2 *b
 // resident in one CTA each; longer ones take the streaming step plus the outer-node rebuild.
 constexpr int kBoundedK = 4;
 constexpr int kBoundedMaxT = 512;
+constexpr int kBoundedMaxTAny = 256;       // CTA size of the FP64 variants with 3, 5 or 6 nodes a thread
 constexpr int kBoundedMaxSteps = 1024;     // steps per resident launch, at most
 constexpr int kBoundedStageBytes = 16384;  // shared memory for the launch's boundary data
 // Dynamic shared memory of k_bounded for a launch of nsteps steps.
@@ -126,12 +127,15 @@ size_t bounded_smem(int b, size_t esz, int nthreads, int D, int nsteps);
 int bounded_launch_steps(int b, size_t esz);
 // Smallest position shift that puts each end's outer nodes and extrapolation node in one warp of
 // the resident kernel (and keeps the instance within one CTA); -1 if there is none.
-int bounded_shift(int b, int N, int depth);
+int bounded_shift(int b, int N, int depth, int K = kBoundedK);
+// Nodes a thread (4, or 3, 5, 6) with which FP64 bounded members of a compiled degree load the SMs'
+// schedulers most evenly.
+int bounded_nodes(int b, const std::vector<lbk::Seg> &m, int sms);
 // dc: the compiled degree (5 on D1Q5, 7 on D1Q7), 0 for a run-time degree, -1 for the variant
 // that also evaluates real-exponent instances (A > 0).
 int launch_bounded(int b, size_t esz, int dc, int ninst, int nthreads, size_t smem, const lbk::BoundedInst *insts_d,
                    const void *in, void *out, const void *coefT, const double *phib, long long stride,
-                   long long step0, int nsteps, cudaStream_t st);
+                   long long step0, int nsteps, cudaStream_t st, int K = kBoundedK);
 int launch_nee_fix(int b, size_t esz, void *st, const lbk::Seg *segs, const int *members, int nmem,
                    const void *coefT, const double *phib, long long stride, long long step, cudaStream_t stream);
 

@@ -106,3 +106,23 @@ def test_fp64_windows(L, eq, sizes64):
         out.append(b.read_phi())
         b.close()
     assert np.isfinite(out[1]).all() and np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("example,count,N,depth", [("4.5", 152, 601, 1), ("4.5", 160, 301, 2), ("4.1", 304, 601, 2), ("4.1", 310, 301, 4),
+                                                   ("4.1", 150, 1530, 1)])
+def test_fp64_bounded_nodes_a_thread(L, example, count, N, depth):
+    """FP64 bounded members on the resident kernel with 3, 4, 5 or 6 nodes a thread, whichever loads
+    the schedulers evenly, against 4 nodes a thread and against the streaming step: equal."""
+    make, ex, dt, tau, scheme, Wd = {"4.1": (W.ks, W.ks_shock, 1e-3, 1.989, 1 | 0x100, 2),
+                                     "4.5": (W.kawahara, W.kawahara_soliton, 1e-4, 2.02, 1, 3)}[example]
+    x = W.grid(-0.05 * (N - 1), N, 0.1)
+    ps = [W.Problem(make(), N, 0.1, dt, tau + 0.002 * i, 0, ex(x, 0.0), xl=x[0], scheme=scheme, boundary="nee", exact_xt=ex,
+                    meta={"depth": depth}) for i in range(count)]
+    pb = W.boundary_values(ps[0], Wd, 0, 60)
+    out = []
+    for args in ((L.KERNEL_AUTO, 0), (L.KERNEL_ONCHIP, 4), (L.KERNEL_STREAM, 0)):
+        b = L.Batch(ps, precision=L.FP64).set_kernel(*args)
+        b.set_phi(np.tile(ps[0].phi0, count)).step_nee(1, pb[:1]).step_nee(59, np.ascontiguousarray(pb[1:]))
+        out.append(b.read_phi())
+        b.close()
+    assert np.isfinite(out[2]).all() and np.array_equal(out[0], out[2]) and np.array_equal(out[1], out[2])
