@@ -891,12 +891,15 @@ void drop_strip(lbhpde_batch_s *bt, Group &g) {
 int plan_strip(lbhpde_batch_s *bt, Group &g, int sms, bool *done) {
     std::vector<Seg> m;
     for (int i : g.members) m.push_back(bt->segs_h[i]);
-    const int dc = lbh::onchip_dc(g.b, g.maxD);
+    const int dc = g.has_nu ? -1 : lbh::onchip_dc(g.b, g.maxD);
+    int AA = 0, DG = 0;
+    *done = false;
+    if (sms <= 0 || !lbh::strip_ok(bt->esz, g.b, dc, m, &AA, &DG)) return LBHPDE_OK;
     lbh::PackedStrip p;
-    if (sms > 0) lbh::pack_strip(g.b, m, p);
+    lbh::pack_strip(g.b, AA, DG, m, p);
     // (the estimate of the other kernels is up to a tenth low where a last wave is half filled:
     // ensembles of 200 and 600 members)
-    *done = sms > 0 && lbh::strip_cost(g.b, p.nwarps(), sms) < 1.1 * lbh::cta_cost(bt->esz, g.b, dc, false, false, m, sms);
+    *done = lbh::strip_cost(g.b, AA, DG, p.nwarps(), sms) < 1.1 * lbh::cta_cost(bt->esz, g.b, dc, false, g.has_nu, m, sms);
     if (!*done) return LBHPDE_OK;
     for (auto &pl : g.ring) {
         bt->dev_free(pl.insts);
@@ -910,7 +913,7 @@ int plan_strip(lbhpde_batch_s *bt, Group &g, int sms, bool *done) {
     g.strip = std::move(p);
     RC(bt->upload(&g.strip_segs, g.strip.segs));
     RC(bt->upload(&g.strip_first, g.strip.first));
-    g.tblk = lbk::strip_steps(g.b);
+    g.tblk = lbk::strip_steps(g.b, g.strip.AA);
     g.onchip_ok = true;
     return LBHPDE_OK;
 }
@@ -1221,7 +1224,7 @@ int choose_kernels(lbhpde_batch_s *bt) {
             sms = 0;
         }
         // strips wherever they are the faster kernel (lbh::strip_cost against lbh::cta_cost)
-        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0 && lbh::strip_ok(bt->esz, g.b, dcg)) {
+        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0) {
             bool done = false;
             RC(plan_strip(bt, g, sms, &done));
             if (done) continue;

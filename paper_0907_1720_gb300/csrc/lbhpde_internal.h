@@ -193,17 +193,19 @@ struct PackedStrip {
     std::vector<lbk::StripSeg> segs;
     std::vector<int> first;
     int b = 0, nfull = 0;
+    int AA = 0, DG = 0;  // row shape of a real-exponent model (AA = 0: polynomial)
     int nmix() const { return first.empty() ? 0 : (int)first.size() - 1; }
     int nwarps() const { return nfull + nmix(); }
 };
-// Whether members of (element size, lattice, on-chip degree code) can take k_strip.
-bool strip_ok(size_t esz, int b, int dc);
-void pack_strip(int b, const std::vector<lbk::Seg> &m, PackedStrip &out);
+// Whether members of (element size, lattice, on-chip degree code) can take k_strip; AA, DG: their row
+// shape (0, 0: polynomials of the compiled degree).
+bool strip_ok(size_t esz, int b, int dc, const std::vector<lbk::Seg> &m, int *AA, int *DG);
+void pack_strip(int b, int AA, int DG, const std::vector<lbk::Seg> &m, PackedStrip &out);
 // What a step costs on a GPU of `sms` SMs, in SM clocks: the CTA-wide kernels on a group's members,
 // k_strip with that many warps.
 double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms);
-double strip_cost(int b, int nwarps, int sms);
-// At most lbk::strip_steps(b) steps, from buffer `in` to another one.
+double strip_cost(int b, int AA, int DG, int nwarps, int sms);
+// At most lbk::strip_steps(b, AA) steps, from buffer `in` to another one.
 int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
                  const void *coefT, int nsteps, cudaStream_t st);
 

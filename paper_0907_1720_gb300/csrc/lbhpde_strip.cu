@@ -9,12 +9,24 @@
 
 namespace lbh {
 
-bool strip_ok(size_t esz, int b, int dc) { return esz == 4 && dc == (b == 5 ? 5 : 7); }
+bool strip_ok(size_t esz, int b, int dc, const std::vector<lbk::Seg> &m, int *AA, int *DG) {
+    *AA = *DG = 0;
+    if (esz != 4 || m.empty()) return false;
+    if (dc >= 0) return dc == (b == 5 ? 5 : 7);
+    // real exponents: one of the compiled row shapes in every member
+    *AA = m[0].A;
+    *DG = m[0].Dg;
+    for (const lbk::Seg &s : m)
+        if (s.A != *AA || s.Dg != *DG) return false;
+    return b == 5 && *AA == 4 && (*DG == 1 || *DG == 5);
+}
 
-void pack_strip(int b, const std::vector<lbk::Seg> &m, PackedStrip &out) {
+void pack_strip(int b, int AA, int DG, const std::vector<lbk::Seg> &m, PackedStrip &out) {
     out = PackedStrip{};
     out.b = b;
-    const int K = lbk::strip_K(b), HL = lbk::strip_HL(b), own = (32 - 2 * HL) * K;
+    out.AA = AA;
+    out.DG = DG;
+    const int K = lbk::strip_K(b, AA), HL = lbk::strip_HL(b), own = (32 - 2 * HL) * K;
     auto seg = [&](const lbk::Seg &s, long long at, int V, int lane0, int nlanes) {
         lbk::StripSeg S{};
         S.off = s.off;
@@ -27,6 +39,7 @@ void pack_strip(int b, const std::vector<lbk::Seg> &m, PackedStrip &out) {
         S.vhi = S.vlo + V;
         S.lane0 = lane0;
         S.nlanes = nlanes;
+        S.nu = (float)s.nu;
         return S;
     };
     struct Rest {
@@ -68,11 +81,11 @@ void pack_strip(int b, const std::vector<lbk::Seg> &m, PackedStrip &out) {
 
 namespace {
 
-template <int B, int DC>
+template <int B, int DC, int AA = 0, int DG = 0>
 int launch_strip_t(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
                    const void *coefT, int nsteps, cudaStream_t st) {
-    auto fn = lbk::k_strip<B, DC>;
-    const int smem = lbk::strip_smem(B, DC);
+    auto fn = lbk::k_strip<B, DC, AA, DG>;
+    const int smem = lbk::strip_smem(B, AA, DC);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         (void)cudaGetLastError();
         return LBHPDE_ERR_CUDA;
@@ -87,7 +100,9 @@ int launch_strip_t(const PackedStrip &p, const lbk::StripSeg *segs, const int *f
 int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
                  const void *coefT, int nsteps, cudaStream_t st) {
     if (p.nwarps() == 0 || nsteps <= 0) return LBHPDE_OK;
-    if (in == out || nsteps > lbk::strip_steps(p.b)) return LBHPDE_ERR_ARG;
+    if (in == out || nsteps > lbk::strip_steps(p.b, p.AA)) return LBHPDE_ERR_ARG;
+    if (p.AA == 4 && p.DG == 1) return launch_strip_t<5, 9, 4, 1>(p, segs, first, in, out, coefT, nsteps, st);
+    if (p.AA == 4 && p.DG == 5) return launch_strip_t<5, 29, 4, 5>(p, segs, first, in, out, coefT, nsteps, st);
     return p.b == 5 ? launch_strip_t<5, 5>(p, segs, first, in, out, coefT, nsteps, st)
                     : launch_strip_t<7, 7>(p, segs, first, in, out, coefT, nsteps, st);
 }

@@ -24,7 +24,7 @@
 //
 // Each node's update is k_onchip's, operation by operation (bit for bit the same results).
 // GB300: 2^24 nodes, 256 steps: D1Q5 9.3e11 node-updates/s (76% of the FP32 pipes; k_onchip's windows
-// 6.2e11), D1Q7 4.7e11 (71%; 3.5e11).
+// 7.0e11), D1Q7 4.6e11 (70%; 3.3e11); u^1.5 u_x (a power and five rows a node) 4.6e11 (3.9e11).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -42,22 +42,26 @@ struct StripSeg {
     int x0;             // node of the segment's position 0 (may be negative: taken modulo N)
     int vlo, vhi;       // own positions [vlo, vhi), written back; vlo = HL K
     int lane0, nlanes;  // lanes [lane0, lane0 + nlanes)
+    float nu;           // real-exponent models: the exponent
 };
 
 constexpr int kStripSegs = 4;  // segments a warp, at most
-__host__ __device__ constexpr int strip_K(int B) { return B == 5 ? 32 : 24; }
+// Models: AA = 0: f^eq of the compiled degree DC; AA > 0: real exponents, P_j = sum_{a<=AA} (phi^nu)^a
+// sum_{i<=DG} c[a (DG + 1) + i] phi^i (D1Q5; the shapes of class (1) with Pi_k = phi).
+__host__ __device__ constexpr int strip_K(int B, int AA) { return B == 5 ? 32 : 24; }
 __host__ __device__ constexpr int strip_HL(int B) { return B == 5 ? 1 : 2; }
 // steps a launch can take: the copies cover steps * max|e| nodes
-__host__ __device__ constexpr int strip_steps(int B) { return strip_HL(B) * strip_K(B) / wmax(B); }
-// shared memory of a warp: the staging rows, then the coefficient rows of its segments
+__host__ __device__ constexpr int strip_steps(int B, int AA) { return strip_HL(B) * strip_K(B, AA) / wmax(B); }
+// shared memory of a warp: the staging rows, then the coefficient rows of its segments (degree D, or
+// (AA + 1)(DG + 1) - 1 for a flattened real-exponent row)
 __host__ __device__ constexpr int strip_pitch(int K) { return K / 4 + 1; }  // 16-byte pieces of a lane
-__host__ __device__ constexpr int strip_smem(int B, int D) {
-    return (B * 32 * strip_pitch(strip_K(B)) * 4 + kStripSegs * cblock(B, D)) * 4;
+__host__ __device__ constexpr int strip_smem(int B, int AA, int D) {
+    return (B * 32 * strip_pitch(strip_K(B, AA)) * 4 + kStripSegs * cblock(B, D)) * 4;
 }
 
 // One step of a lane's K nodes: pull from its own registers and the lanes beside it, phi, relaxation.
-template <int B, int DC, int K, int CH>
-__device__ __forceinline__ void strip_step(float (&phi)[K], float (&v)[B - 1][K], const float *c0, float omw) {
+template <int B, int DC, int AA, int DG, int K, int CH>
+__device__ __forceinline__ void strip_step(float (&phi)[K], float (&v)[B - 1][K], const float *c0, float omw, float nu) {
     constexpr int CS = crow(DC);
     float d[K];
 #pragma unroll
@@ -96,6 +100,11 @@ __device__ __forceinline__ void strip_step(float (&phi)[K], float (&v)[B - 1][K]
         const float2 p2 = __fadd2_rn(make_float2(phi[k], phi[k + 1]), make_float2(d[k], d[k + 1]));
         phi[k] = p2.x, phi[k + 1] = p2.y;
     }
+    float wp[AA > 0 ? K : 1];  // phi^nu
+    if constexpr (AA > 0) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) wp[k] = nu_pow<float>(phi[k], nu);
+    }
     // A right-moving population relaxes from its last node down, a left-moving one from its first
     // node up: node k's new value may then take the register that held k before the pull, whose old
     // value (a neighbour's source) has been used.  In ascending order for all, a move a node went
@@ -107,15 +116,36 @@ __device__ __forceinline__ void strip_step(float (&phi)[K], float (&v)[B - 1][K]
         for (int b0 = 0; b0 < K; b0 += CH) {
             const int i0 = vel(j) > 0 ? K - CH - b0 : b0;
             float2 acc[CH / 2];
-            const float cD = c[DC];
+            if constexpr (AA == 0) {
+                const float cD = c[DC];
 #pragma unroll
-            for (int i = 0; i < CH / 2; ++i) acc[i] = make_float2(cD, cD);
+                for (int i = 0; i < CH / 2; ++i) acc[i] = make_float2(cD, cD);
 #pragma unroll
-            for (int p = DC - 1; p >= 0; --p) {
-                const float cp = c[p];
+                for (int p = DC - 1; p >= 0; --p) {
+                    const float cp = c[p];
 #pragma unroll
-                for (int i = 0; i < CH / 2; ++i)
-                    acc[i] = __ffma2_rn(acc[i], make_float2(phi[i0 + 2 * i], phi[i0 + 2 * i + 1]), make_float2(cp, cp));
+                    for (int i = 0; i < CH / 2; ++i)
+                        acc[i] = __ffma2_rn(acc[i], make_float2(phi[i0 + 2 * i], phi[i0 + 2 * i + 1]), make_float2(cp, cp));
+                }
+            } else {
+                // Horner in phi within a row, in w = phi^nu across rows (as gen_evalN)
+#pragma unroll
+                for (int a = AA; a >= 0; --a) {
+                    float2 h[CH / 2];
+                    const float cD = c[a * (DG + 1) + DG];
+#pragma unroll
+                    for (int i = 0; i < CH / 2; ++i) h[i] = make_float2(cD, cD);
+#pragma unroll
+                    for (int p = DG - 1; p >= 0; --p) {
+                        const float cp = c[a * (DG + 1) + p];
+#pragma unroll
+                        for (int i = 0; i < CH / 2; ++i)
+                            h[i] = __ffma2_rn(h[i], make_float2(phi[i0 + 2 * i], phi[i0 + 2 * i + 1]), make_float2(cp, cp));
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH / 2; ++i)
+                        acc[i] = a == AA ? h[i] : __ffma2_rn(acc[i], make_float2(wp[i0 + 2 * i], wp[i0 + 2 * i + 1]), h[i]);
+                }
             }
 #pragma unroll
             for (int h = 0; h < CH / 2; ++h) {
@@ -129,13 +159,13 @@ __device__ __forceinline__ void strip_step(float (&phi)[K], float (&v)[B - 1][K]
     }
 }
 
-template <int B, int DC>
+template <int B, int DC, int AA = 0, int DG = 0>
 __global__ void __launch_bounds__(32, 8)
     k_strip(const float *__restrict__ st_in, float *__restrict__ st_out, const StripSeg *__restrict__ segs,
             const int *__restrict__ first, int nmix, const float *__restrict__ coefs, int nsteps) {
-    constexpr int K = strip_K(B), KQ = K / 4, PQ = strip_pitch(K);
+    constexpr int K = strip_K(B, AA), KQ = K / 4, PQ = strip_pitch(K);
     constexpr int CS = crow(DC), CB = cblock(B, DC);
-    constexpr int CH = 4;  // nodes a Horner chunk (8 to 32: equal or 1% slower)
+    constexpr int CH = AA > 0 ? 8 : 4;  // nodes a Horner chunk (others: equal or 1% slower)
     static_assert(K % CH == 0 && CH % 2 == 0 && K <= 32, "packed pairs; a node a lane where a lane's nodes are moved singly");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *const stage = reinterpret_cast<float4 *>(smem_raw);  // [B][32][PQ]
@@ -174,6 +204,7 @@ __global__ void __launch_bounds__(32, 8)
     };
     float phi[K], v[B - 1][K];
     int mine;
+    float nu = 1.f;
     {
     const Place pl = place(0);
     mine = pl.mine;
@@ -194,6 +225,7 @@ __global__ void __launch_bounds__(32, 8)
         }
     }
     const int s0 = w < nmix ? first[w] : w - nmix, ns = w < nmix ? first[w + 1] - s0 : 1;
+    if (AA > 0 && mine >= 0) nu = segs[s0 + mine].nu;
     for (int s = 0; s < ns; ++s) {  // (while the state is under way)
         const StripSeg &S = segs[s0 + s];
         for (int q = lane; q < (B - 1) * CS; q += 32) {
@@ -238,7 +270,7 @@ __global__ void __launch_bounds__(32, 8)
     const float omw = c0[(B - 1) * CS];
 
 #pragma unroll 1
-    for (int s = 0; s < nsteps; ++s) strip_step<B, DC, K, CH>(phi, v, c0, omw);
+    for (int s = 0; s < nsteps; ++s) strip_step<B, DC, AA, DG, K, CH>(phi, v, c0, omw, nu);
 
     // own positions of the lane: [lo, hi) of its K; whole 16-byte pieces go out coalesced, the rest
     // (a lane that wraps or is not aligned, an own range that ends inside a piece) node by node

@@ -294,8 +294,9 @@ double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vecto
 
 // A step of k_strip: one warp on a scheduler, two, and every further wave of two (GB300: D1Q5 400 000
 // nodes 2160, 800 000 3440, 2^24 37 800; D1Q7 400 000 2840, 800 000 4800, 2^24 75 400).
-double strip_cost(int b, int nwarps, int sms) {
-    const double one = b == 5 ? 2100 : 2840, two = b == 5 ? 3440 : 4800, more = b == 5 ? 2570 : 3620;
+double strip_cost(int b, int AA, int DG, int nwarps, int sms) {
+    const double s = AA > 0 ? (DG == 1 ? 2.0 : 4.9) : 1.0;  // the power and the rows (2^24 nodes: 76 000 and 180 000)
+    const double one = s * (b == 5 ? 2100 : 2840), two = s * (b == 5 ? 3440 : 4800), more = s * (b == 5 ? 2570 : 3620);
     const double waves = nwarps / (8.0 * sms);
     if (waves <= 0.5) return one;
     if (waves <= 1.0) return two;
@@ -349,10 +350,11 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
     }
     std::stable_sort(picks.begin(), picks.end(), [](const WavePick &x, const WavePick &y) { return x.cost < y.cost; });
     double other = cta_cost(esz, b, dc, nee, real, m, sms);
-    if (!nee && strip_ok(esz, b, dc)) {
+    int AA = 0, DG = 0;
+    if (!nee && strip_ok(esz, b, dc, m, &AA, &DG)) {
         PackedStrip p;
-        pack_strip(b, m, p);
-        other = std::min(other, strip_cost(b, p.nwarps(), sms));
+        pack_strip(b, AA, DG, m, p);
+        other = std::min(other, strip_cost(b, AA, DG, p.nwarps(), sms));
     }
     for (const WavePick &k : picks) {
         if (k.cost > 0.85 * other) return false;

@@ -23,7 +23,8 @@ int main() {
     std::mt19937 g(11);
     size_t warps = 0, lanes = 0, own = 0;
     for (int t = 0; t < 200 && !fails; ++t) {
-        const int b = g() % 2 ? 5 : 7, W = lbk::wmax(b), K = lbk::strip_K(b), P = 32 * K, T = lbk::strip_steps(b);
+        const int b = g() % 2 ? 5 : 7, W = lbk::wmax(b), AA = b == 5 && g() % 2 ? 4 : 0;
+        const int K = lbk::strip_K(b, AA), P = 32 * K, T = lbk::strip_steps(b, AA);
         std::vector<lbk::Seg> m;
         for (int i = 0, n = 1 + (int)(g() % 40); i < n; ++i) {
             lbk::Seg s{};
@@ -33,7 +34,7 @@ int main() {
             m.push_back(s);
         }
         lbh::PackedStrip p;
-        lbh::pack_strip(b, m, p);
+        lbh::pack_strip(b, AA, AA ? 1 : 0, m, p);
         std::vector<std::vector<int>> count(m.size());
         for (size_t i = 0; i < m.size(); ++i) count[i].assign(m[i].N, 0);
         for (int w = 0; w < p.nwarps(); ++w) {

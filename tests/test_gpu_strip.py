@@ -25,6 +25,8 @@ def L():
 
 
 EQS = {"kdv": (lambda i: W.kdv_burgers(1.0 + 0.2 * i % 5, 0.01 * (i % 9), 0.5 + 0.01 * (i % 50)), 1e-4, 1.15),
+       "gkdv": (lambda i: W.gkdv(1.5 + 0.01 * (i % 7)), 1e-4, 1.3),
+       "class1": (lambda i: W.class1_real(0.5, 1.0, 1.5, (0.0, 1.0)), 1e-4, 1.3),
        "kawahara": (lambda i: W.kawahara(1.0, 0.5 + 0.01 * (i % 50), -1.0), 1e-4, 2.02)}
 
 
@@ -40,7 +42,7 @@ def members(eq, sizes):
 
 def sizes(own, K):
     edge = [6, 7, 31, K - 1, K, K + 1, own - 1, own, own + 1, own + K + 3, 2 * own, 2 * own + 5, 4099]
-    return edge + list(np.random.default_rng(own).integers(256, 8193, 700))
+    return edge + list(np.random.default_rng(own).integers(256, 8193, 1000))
 
 
 def solve(L, ps, kernel, calls):
@@ -56,7 +58,7 @@ def solve(L, ps, kernel, calls):
     return out, launches
 
 
-@pytest.mark.parametrize("eq,own,K", [("kdv", 960, 32), ("kawahara", 672, 24)])
+@pytest.mark.parametrize("eq,own,K", [("kdv", 960, 32), ("kawahara", 672, 24), ("gkdv", 960, 32)])
 def test_batch(L, eq, own, K):
     ps = members(eq, sizes(own, K))
     a, n = solve(L, ps, L.KERNEL_AUTO, [1, 15, 16, 17, 33])
@@ -65,7 +67,7 @@ def test_batch(L, eq, own, K):
     assert np.isfinite(b).all() and np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("eq,N", [("kdv", (1 << 22) + 3), ("kawahara", (1 << 21) + 1)])
+@pytest.mark.parametrize("eq,N", [("kdv", (1 << 22) + 3), ("kawahara", (1 << 21) + 1), ("gkdv", (1 << 22) + 1), ("class1", (1 << 22) + 2)])
 def test_long_grid(L, eq, N):
     ps = members(eq, [N])
     a, n = solve(L, ps, L.KERNEL_AUTO, [40])
