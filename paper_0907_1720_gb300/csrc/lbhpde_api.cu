@@ -295,7 +295,11 @@ int default_tblk(int capacity, int W, int valid_eighths) {
     return t;
 }
 
-int onchip_dc(int b, int maxD) { return maxD == (b == 5 ? 5 : 7) ? maxD : 0; }
+int onchip_dc(int b, int maxD) {
+    // D1Q5: 5 (a quadratic flux) and 9 (a cubic one, and the degrees between); D1Q7: 7
+    if (b == 5) return maxD == 5 ? 5 : (maxD > 5 && maxD <= 9 ? 9 : 0);
+    return maxD == 7 ? 7 : 0;
+}
 
 bool split_ring_waves(int b, int K, int sms, const std::vector<Member> &m, std::vector<Member> &full,
                       std::vector<Member> &tail) {

@@ -193,12 +193,12 @@ struct PackedStrip {
     std::vector<lbk::StripSeg> segs;
     std::vector<int> first;
     int b = 0, nfull = 0;
-    int AA = 0, DG = 0;  // row shape of a real-exponent model (AA = 0: polynomial)
+    int AA = 0, DG = 0;  // row shape of a real-exponent model (AA = 0: polynomials, of compiled degree DG)
     int nmix() const { return first.empty() ? 0 : (int)first.size() - 1; }
     int nwarps() const { return nfull + nmix(); }
 };
 // Whether members of (element size, lattice, on-chip degree code) can take k_strip; AA, DG: their row
-// shape (0, 0: polynomials of the compiled degree).
+// shape (AA = 0: polynomials, of compiled degree DG).
 bool strip_ok(size_t esz, int b, int dc, const std::vector<lbk::Seg> &m, int *AA, int *DG);
 void pack_strip(int b, int AA, int DG, const std::vector<lbk::Seg> &m, PackedStrip &out);
 // What a step costs on a GPU of `sms` SMs, in SM clocks: the CTA-wide kernels on a group's members,

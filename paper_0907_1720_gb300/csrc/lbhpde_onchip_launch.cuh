@@ -45,11 +45,14 @@ int launch_onchip_t(const OnchipArgs &a) {
 }
 
 // compile-time polynomial degree: D = 5 on D1Q5 and D = 7 on D1Q7 (the KdV/KS/KdV-Burgers and
-// Kawahara families), run-time degree otherwise
+// Kawahara families), D = 9 on D1Q5 (mKdV), run-time degree otherwise
 template <typename T, int B, int K, int MAXT, bool HALO>
 int launch_onchip_d(int dc, const OnchipArgs &a) {
     constexpr int DC = B == 5 ? 5 : 7;
     if (dc == DC) return launch_onchip_t<T, B, K, MAXT, HALO, DC>(a);
+    // a cubic flux: 8 nodes a thread in FP32 (elsewhere the run-time degree serves it)
+    if constexpr (sizeof(T) == 4 && B == 5 && K == 8)
+        if (dc == 9) return launch_onchip_t<T, B, K, MAXT, HALO, 9>(a);
     if (dc < 0) {  // real exponents: evaluated four nodes at a time, so K >= 4
         if constexpr (K >= 4) return launch_onchip_t<T, B, K, MAXT, HALO, -1>(a);
         return LBHPDE_ERR_UNSUPPORTED;

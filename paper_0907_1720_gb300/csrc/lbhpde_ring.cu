@@ -31,7 +31,7 @@ template <int MAXT>
 int launch_ring_d(int dc, const Packed &p, const lbk::OnchipInst *insts, const int *first, const void *in, void *out,
                   const void *coefT, int nsteps, cudaStream_t st) {
     if (dc == 5) return launch_ring_t<MAXT, 5>(p, insts, first, in, out, coefT, nsteps, st);
-    if (dc == 0) return launch_ring_t<MAXT, 0>(p, insts, first, in, out, coefT, nsteps, st);
+    if (dc >= 0) return launch_ring_t<MAXT, 0>(p, insts, first, in, out, coefT, nsteps, st);
     return LBHPDE_ERR_UNSUPPORTED;
 }
 
@@ -72,9 +72,9 @@ int launch_ring_nee_d(int dc, const PackedNee &p, const lbk::RingNeeInst *insts,
     if (dc == 5 && p.d2)
         return launch_ring_nee_t<MAXT, 5, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
     if (dc == 5) return launch_ring_nee_t<MAXT, 5, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
-    if (dc == 0 && p.d2)
+    if (dc >= 0 && p.d2)
         return launch_ring_nee_t<MAXT, 0, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
-    if (dc == 0) return launch_ring_nee_t<MAXT, 0, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
+    if (dc >= 0) return launch_ring_nee_t<MAXT, 0, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
     return LBHPDE_ERR_UNSUPPORTED;
 }
 

@@ -12,7 +12,10 @@ namespace lbh {
 bool strip_ok(size_t esz, int b, int dc, const std::vector<lbk::Seg> &m, int *AA, int *DG) {
     *AA = *DG = 0;
     if (esz != 4 || m.empty()) return false;
-    if (dc >= 0) return dc == (b == 5 ? 5 : 7);
+    if (dc >= 0) {
+        *DG = dc;
+        return dc == (b == 5 ? 5 : 7) || (b == 5 && dc == 9);
+    }
     // real exponents: one of the compiled row shapes in every member
     *AA = m[0].A;
     *DG = m[0].Dg;
@@ -103,6 +106,7 @@ int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *fir
     if (in == out || nsteps > lbk::strip_steps(p.b, p.AA)) return LBHPDE_ERR_ARG;
     if (p.AA == 4 && p.DG == 1) return launch_strip_t<5, 9, 4, 1>(p, segs, first, in, out, coefT, nsteps, st);
     if (p.AA == 4 && p.DG == 5) return launch_strip_t<5, 29, 4, 5>(p, segs, first, in, out, coefT, nsteps, st);
+    if (p.b == 5 && p.DG == 9) return launch_strip_t<5, 9>(p, segs, first, in, out, coefT, nsteps, st);
     return p.b == 5 ? launch_strip_t<5, 5>(p, segs, first, in, out, coefT, nsteps, st)
                     : launch_strip_t<7, 7>(p, segs, first, in, out, coefT, nsteps, st);
 }

@@ -73,6 +73,8 @@ template <typename T, int B, int K, int G, bool NEE>
 int launch_wave_d(const WaveArgs &a) {
     constexpr int DC = B == 5 ? 5 : 7;
     if (a.p->dc == DC) return launch_wave_t<T, B, K, G, DC, NEE>(a);
+    if constexpr (B == 5)
+        if (a.p->dc == 9) return launch_wave_t<T, B, K, G, 9, NEE>(a);
     if constexpr (K == (sizeof(T) == 4 ? 2 : 1) && G == 1) {  // run-time degrees and real exponents
         if (a.p->dc == 0) return launch_wave_t<T, B, K, G, 0, NEE>(a);
         if (a.p->dc < 0) return launch_wave_t<T, B, K, G, -1, NEE>(a);
@@ -285,7 +287,9 @@ double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vecto
     double all = (resident + windows) * ops / (rate * sms);
     if (esz == 4 && !nee) {
         const double waves = resident / (512.0 * kRingK * sms), rest = waves - (long long)waves;
-        const double res = ring ? 3400 * ((long long)waves + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0))) : resident * ops / (60.0 * sms);
+        // (a degree k_ring has not compiled takes single multiply-adds)
+        const double wave = 3400 * ops / wave_ops(5, 5) * (dc == 5 ? 1.0 : 1.5);
+        const double res = ring ? wave * ((long long)waves + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0))) : resident * ops / (60.0 * sms);
         const double win = windows == 0 ? 0 : (b == 5 ? 450 + windows * ops / (66.0 * sms) : 1840 * std::ceil(windows / (1856.0 * sms)) * ops / wave_ops(7, 7));
         all = res + win;
     }
@@ -295,7 +299,7 @@ double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vecto
 // A step of k_strip: one warp on a scheduler, two, and every further wave of two (GB300: D1Q5 400 000
 // nodes 2160, 800 000 3440, 2^24 37 800; D1Q7 400 000 2840, 800 000 4800, 2^24 75 400).
 double strip_cost(int b, int AA, int DG, int nwarps, int sms) {
-    const double s = AA > 0 ? (DG == 1 ? 2.0 : 4.9) : 1.0;  // the power and the rows (2^24 nodes: 76 000 and 180 000)
+    const double s = AA > 0 ? (DG == 1 ? 2.0 : 4.9) : wave_ops(b, DG) / wave_ops(b, b == 5 ? 5 : 7);  // the power and the rows (2^24 nodes: 76 000 and 180 000)
     const double one = s * (b == 5 ? 2100 : 2840), two = s * (b == 5 ? 3440 : 4800), more = s * (b == 5 ? 2570 : 3620);
     const double waves = nwarps / (8.0 * sms);
     if (waves <= 0.5) return one;

@@ -34,7 +34,7 @@ int main() {
             m.push_back(s);
         }
         lbh::PackedStrip p;
-        lbh::pack_strip(b, AA, AA ? 1 : 0, m, p);
+        lbh::pack_strip(b, AA, AA ? 1 : (b == 5 ? 5 : 7), m, p);
         std::vector<std::vector<int>> count(m.size());
         for (size_t i = 0; i < m.size(); ++i) count[i].assign(m[i].N, 0);
         for (int w = 0; w < p.nwarps(); ++w) {

@@ -25,6 +25,7 @@ def L():
 
 
 EQS = {"kdv": (lambda i: W.kdv_burgers(1.0 + 0.2 * i % 5, 0.01 * (i % 9), 0.5 + 0.01 * (i % 50)), 1e-4, 1.15),
+       "mkdv": (lambda i: W.mkdv(), 1e-5, 1.2),  # degree 9
        "gkdv": (lambda i: W.gkdv(1.5 + 0.01 * (i % 7)), 1e-4, 1.3),
        "class1": (lambda i: W.class1_real(0.5, 1.0, 1.5, (0.0, 1.0)), 1e-4, 1.3),
        "kawahara": (lambda i: W.kawahara(1.0, 0.5 + 0.01 * (i % 50), -1.0), 1e-4, 2.02)}
@@ -46,7 +47,11 @@ def sizes(own, K):
 
 
 def solve(L, ps, kernel, calls):
-    b = L.Batch(ps, precision=L.FP32_DEV).set_kernel(kernel)
+    return solve_k(L, ps, (kernel, 0), calls)
+
+
+def solve_k(L, ps, kernel, calls):
+    b = L.Batch(ps, precision=L.FP32_DEV).set_kernel(*kernel)
     b.set_phi(np.concatenate([p.phi0 for p in ps]))
     launches = []
     for n in calls:
@@ -58,7 +63,7 @@ def solve(L, ps, kernel, calls):
     return out, launches
 
 
-@pytest.mark.parametrize("eq,own,K", [("kdv", 960, 32), ("kawahara", 672, 24), ("gkdv", 960, 32)])
+@pytest.mark.parametrize("eq,own,K", [("kdv", 960, 32), ("kawahara", 672, 24), ("mkdv", 960, 32), ("gkdv", 960, 32)])
 def test_batch(L, eq, own, K):
     ps = members(eq, sizes(own, K))
     a, n = solve(L, ps, L.KERNEL_AUTO, [1, 15, 16, 17, 33])
@@ -73,6 +78,15 @@ def test_long_grid(L, eq, N):
     a, n = solve(L, ps, L.KERNEL_AUTO, [40])
     b, _ = solve(L, ps, L.KERNEL_STREAM, [40])
     assert n == [3] and np.array_equal(a, b)
+
+
+def test_cubic_flux_on_chip(L):
+    """Degree 9 compiled into the on-chip kernel (resident and windows, every CTA class), equal to the
+    streaming kernel's run-time degree."""
+    ps = members("mkdv", [6, 500, 1000, 1025, 2047, 4000, 4097, 9001])
+    a, _ = solve_k(L, ps, (L.KERNEL_ONCHIP, 8), [1, 39])
+    b, _ = solve_k(L, ps, (L.KERNEL_STREAM, 0), [40])
+    assert np.isfinite(b).all() and np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("steps", [1, 16, 40])
