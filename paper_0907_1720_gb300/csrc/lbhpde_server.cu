@@ -152,7 +152,7 @@ struct DevBuf {  // growable device array (capacity only grows)
 struct lbhpde_server_s {
     int precision = LBHPDE_FP32_DEV;
     size_t esz = 4;
-    int device = 0, max_active = 0, block = 256;
+    int device = 0, max_active = 0, block = 256, sms = 0;
     cudaStream_t stream = nullptr;
     // set-up of admitted requests (uploads, initialisation) runs on `up`, beside a block in
     // flight on `stream`; `stream` waits for it through ev_setup
@@ -384,6 +384,14 @@ int plan_block(lbhpde_server_s *S, Block &blk) {
     blk = Block{};
     blk.id = S->next_block;
     std::vector<Planned> &plan = blk.plan;
+    // FP32 windows of 128 threads (1024 nodes, 32 steps a launch) while the requests in flight leave
+    // SMs idle, of a resident CTA's size otherwise, when the wider ones' smaller share of copies counts
+    // (GB300, ms a burst, wide and narrow: 8 requests 8.0 and 5.0, 12 5.2 and 3.1, 24 with 279 000 nodes
+    // 9.6 and 6.3; 48 with 558 000 nodes 13.7 and 14.6, 200 29.9 and 32.4)
+    long long in_flight = 0;
+    for (const Req *r : S->active)
+        if (r->done < r->nsteps) in_flight += r->N;
+    const bool narrow = S->esz == 4 && in_flight < 2000LL * S->sms;
     // per lattice, three classes: requests whose f^eq degree the compiled variant covers (D <= 5
     // on D1Q5, <= 7 on D1Q7), higher-degree polynomials, and real-exponent models, each with its
     // own launches, so that one high-degree or real-exponent request does not send the whole
@@ -395,7 +403,7 @@ int plan_block(lbhpde_server_s *S, Block &blk) {
         const int K = lbh::default_K(S->esz, b);
         const int maxt = lbh::onchip_maxt(S->esz, b, K);
         const int cap = maxt * K, W = (b - 1) / 2;
-        const int tblk = lbh::default_tblk(cap, W, 6);  // windows as wide as a resident CTA
+        int tblk = narrow ? 32 : lbh::default_tblk(cap, W, 6), wthr = narrow ? 128 : 0;
         // resident requests keep the windows' K: a request's latency is set by its own CTA, and
         // more threads an instance hold its steps shorter when the GPU is not full (the 16-node
         // kernel gave the same throughput at 2000 requests/s on GB300, and 0.35 s against
@@ -418,6 +426,21 @@ int plan_block(lbhpde_server_s *S, Block &blk) {
         if (!bnd.empty()) SRC(plan_bounded(S, blk, b, kind, maxDb, bnd));
         if (ring.empty() && halo.empty()) continue;
         const int dc = kind == 2 ? -1 : lbh::onchip_dc(b, maxD);
+        // FP64: windows of the size and depth that load the SMs evenly, for the short requests too where
+        // that is faster (as batches)
+        if (S->esz == 8 && kind != 2) {
+            std::vector<Seg> segs;
+            for (const auto *v : {&ring, &halo})
+                for (const Req *r : *v) segs.push_back(r->seg());
+            int T = 0;
+            if (lbh::windows_f64(b, dc, K, segs, S->sms, &wthr, &T)) {
+                tblk = T;
+                halo.insert(halo.end(), ring.begin(), ring.end());
+                ring.clear();
+            } else {
+                wthr = 0;
+            }
+        }
         if (!ring.empty()) {
             std::vector<lbh::Member> m;
             int n = 0;
@@ -457,7 +480,7 @@ int plan_block(lbhpde_server_s *S, Block &blk) {
                 }
                 if (m.empty()) break;
                 Planned pl{b, K, dc, true, 4 * cls + 3, n, {}};
-                SRC(lbh::pack_halo(b, S->esz, K, dc, tblk * W, m, pl.p, true));
+                SRC(lbh::pack_halo(b, S->esz, K, dc, tblk * W, m, pl.p, true, wthr));
                 plan.push_back(std::move(pl));
             }
         }
@@ -739,6 +762,7 @@ extern "C" int lbhpde_server_create(lbhpde_server_t *out, int precision, size_t 
     S->t0 = Clock::now();
     int prev = 0;
     bool ok = cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(device) == cudaSuccess &&
+              cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, device) == cudaSuccess &&
               cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&S->up, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&S->ev_setup, cudaEventDisableTiming) == cudaSuccess &&
