@@ -821,7 +821,10 @@ __global__ void __launch_bounds__(MAXT, onchip_minb(sizeof(T), B, K, MAXT))
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < K; ++k) v[j][k] = fma_t(omw, v[j][k], acc[k]);
+                for (int h = 0; h < K; ++h) {  // (towards the side the population came from: no register moves)
+                    const int k = vel(j) > 0 ? K - 1 - h : h;
+                    v[j][k] = fma_t(omw, v[j][k], acc[k]);
+                }
             }
         }
     }

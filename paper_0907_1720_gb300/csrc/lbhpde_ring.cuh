@@ -67,7 +67,8 @@ __device__ __forceinline__ void ring_relax(const T *sc, int cs, int D, T omw, co
             if constexpr (DC > 0 && std::is_same<T, float>::value && CH % 2 == 0 && NN % CH == 0) {
                 // two nodes per packed FP32 multiply-add (the same roundings as one at a time)
 #pragma unroll
-                for (int i0 = 0; i0 < NN; i0 += CH) {
+                for (int b0 = 0; b0 < NN; b0 += CH) {
+                    const int i0 = vel(j) > 0 ? NN - CH - b0 : b0;
                     float2 acc[CH / 2];
                     const float cD = c[DC];
 #pragma unroll
@@ -81,9 +82,11 @@ __device__ __forceinline__ void ring_relax(const T *sc, int cs, int D, T omw, co
                             acc[i] = __ffma2_rn(acc[i], make_float2(phi[node(i0 + 2 * i)], phi[node(i0 + 2 * i + 1)]), cp2);
                     }
 #pragma unroll
-                    for (int i = 0; i < CH / 2; ++i) {
-                        v[j][node(i0 + 2 * i)] = fma_t(omw, v[j][node(i0 + 2 * i)], acc[i].x);
-                        v[j][node(i0 + 2 * i + 1)] = fma_t(omw, v[j][node(i0 + 2 * i + 1)], acc[i].y);
+                    for (int h = 0; h < CH / 2; ++h) {
+                        const int i = vel(j) > 0 ? CH / 2 - 1 - h : h, n0 = node(i0 + 2 * i), n1 = node(i0 + 2 * i + 1);
+                        if (vel(j) > 0) v[j][n1] = fma_t(omw, v[j][n1], acc[i].y);
+                        v[j][n0] = fma_t(omw, v[j][n0], acc[i].x);
+                        if (vel(j) < 0) v[j][n1] = fma_t(omw, v[j][n1], acc[i].y);
                     }
                 }
             } else if constexpr (DC > 0) {

@@ -328,9 +328,12 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
                         for (int k = 0; k < K / 2; ++k)
                             a2[k] = __ffma2_rn(a2[k], make_float2(phi[2 * k], phi[2 * k + 1]), make_float2(c[i][p], c[i][p]));
 #pragma unroll
-                    for (int k = 0; k < K / 2; ++k) {
+                    for (int h = 0; h < K / 2; ++h) {
+                        const bool right = G == 1 && vel(1 + i) > 0;
+                        const int k = right ? K / 2 - 1 - h : h;
+                        if (right) v[i][2 * k + 1] = fma_t(omw, v[i][2 * k + 1], a2[k].y);
                         v[i][2 * k] = fma_t(omw, v[i][2 * k], a2[k].x);
-                        v[i][2 * k + 1] = fma_t(omw, v[i][2 * k + 1], a2[k].y);
+                        if (!right) v[i][2 * k + 1] = fma_t(omw, v[i][2 * k + 1], a2[k].y);
                     }
                 } else {
                     T acc[K];
