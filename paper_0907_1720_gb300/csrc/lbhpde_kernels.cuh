@@ -821,8 +821,10 @@ __global__ void __launch_bounds__(MAXT, onchip_minb(sizeof(T), B, K, MAXT))
                     }
                 }
 #pragma unroll
-                for (int h = 0; h < K; ++h) {  // (towards the side the population came from: no register moves)
-                    const int k = vel(j) > 0 ? K - 1 - h : h;
+                for (int h = 0; h < K; ++h) {
+                    // FP32: towards the side the population came from, which saves register moves
+                    // (4%); FP64 D1Q7 windows are 10% slower that way
+                    const int k = sizeof(T) == 4 && vel(j) > 0 ? K - 1 - h : h;
                     v[j][k] = fma_t(omw, v[j][k], acc[k]);
                 }
             }
