@@ -19,8 +19,8 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(BUILD, "liblbhpde.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["lbhpde_model.cpp", "lbhpde_api.cu", "lbhpde_onchip_f32.cu", "lbhpde_onchip_f64.cu", "lbhpde_ring.cu",
-           "lbhpde_bounded.cu", "lbhpde_wave_f32.cu", "lbhpde_wave_f64.cu", "lbhpde_strip.cu", "lbhpde_noalloc.cu", "lbhpde_server.cu"]
-HEADERS = ["lbhpde_kernels.cuh", "lbhpde_bounded.cuh", "lbhpde_ring.cuh", "lbhpde_ring_nee.cuh", "lbhpde_wave.cuh", "lbhpde_wave_launch.cuh", "lbhpde_strip.cuh", "lbhpde_internal.h", "lbhpde_onchip_launch.cuh"]
+           "lbhpde_bounded.cu", "lbhpde_wave_f32.cu", "lbhpde_wave_f64.cu", "lbhpde_strip.cu", "lbhpde_span.cu", "lbhpde_noalloc.cu", "lbhpde_server.cu"]
+HEADERS = ["lbhpde_kernels.cuh", "lbhpde_bounded.cuh", "lbhpde_ring.cuh", "lbhpde_ring_nee.cuh", "lbhpde_wave.cuh", "lbhpde_wave_launch.cuh", "lbhpde_strip.cuh", "lbhpde_span.cuh", "lbhpde_internal.h", "lbhpde_onchip_launch.cuh"]
 
 
 def _nvcc():

@@ -80,6 +80,9 @@ struct Group {
     lbk::RingNeeInst *rn_insts = nullptr;
     int *rn_first = nullptr;
     int rn_dc = 0;
+    std::vector<lbk::SpanInst> sp_h;   // bounded members of one warp each, by nodes a lane
+    std::vector<std::pair<int, int>> sp_first;  // (nodes a lane, first of its members), in order
+    lbk::SpanInst *sp = nullptr;
     std::vector<int> smembers_h;       // streaming members
     int *smembers = nullptr;
     std::vector<int2> sblocks_h;       // their node blocks (kChunk nodes each)
@@ -1060,6 +1063,8 @@ int batch_build(lbhpde_batch_s *bt, int count, const lbhpde_instance *m) {
 // (unless the streaming kernel was requested); longer ones stream and are rebuilt each step.
 int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.bnd_h.clear();
+    g.sp_h.clear();
+    g.sp_first.clear();
     g.smembers_h.clear();
     g.sblocks_h.clear();
     int K = lbh::kBoundedK;
@@ -1076,13 +1081,25 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.bnd_K = K;
     int maxthr = 0, maxD = 0, maxDn = 0;
     bool real = false;
-    // FP32 D1Q5 polynomial members take the 16-node resident kernel (unless a kernel or 4 nodes
-    // a thread was asked for), the others one CTA each (real-exponent members on its variant
-    // with the generalised f^eq) or the streaming step
+    // FP32 D1Q5 polynomial members take a warp each where lbh::span_ok says so (automatic choice),
+    // else the 16-node resident kernel (unless a kernel or 4 nodes a thread was asked for), the
+    // others one CTA each (real-exponent members on its variant with the generalised f^eq) or the
+    // streaming step
     std::vector<lbh::NeeMember> nee;
     const bool nee_auto = bt->kernel == LBHPDE_KERNEL_AUTO || (bt->kernel == LBHPDE_KERNEL_ONCHIP && bt->K_req != K4);
     for (int i : g.members) {
         const Seg &sg = bt->segs_h[i];
+        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && lbh::span_ok(bt->esz, g.b, sg)) {
+            lbk::SpanInst I{};
+            I.off = sg.off;
+            I.ld = sg.ld;
+            I.N = sg.N;
+            I.D = sg.D;
+            I.gcoef = sg.coef;
+            I.mi = i;
+            g.sp_h.push_back(I);
+            continue;
+        }
         if (nee_auto && lbh::ring_nee_ok(bt->esz, g.b, sg)) {
             nee.push_back(lbh::NeeMember{sg, i, 1 << 30});
             maxDn = std::max(maxDn, sg.D);
@@ -1121,6 +1138,8 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     bt->dev_free(g.sblocks);
     bt->dev_free(g.rn_insts);
     bt->dev_free(g.rn_first);
+    bt->dev_free(g.sp);
+    g.sp = nullptr;
     g.bnd = nullptr;
     g.smembers = nullptr;
     g.sblocks = nullptr;
@@ -1133,6 +1152,14 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
         RC(bt->upload(&g.rn_insts, g.rn_h.insts));
         RC(bt->upload(&g.rn_first, g.rn_h.first));
     }
+    if (!g.sp_h.empty()) {
+        std::stable_sort(g.sp_h.begin(), g.sp_h.end(),
+                         [](const lbk::SpanInst &x, const lbk::SpanInst &y) { return lbh::span_nodes(x.N) > lbh::span_nodes(y.N); });
+        for (size_t q = 0; q < g.sp_h.size(); ++q)  // a launch for each number of nodes a lane
+            if (q == 0 || lbh::span_nodes(g.sp_h[q].N) != g.sp_first.back().first)
+                g.sp_first.emplace_back(lbh::span_nodes(g.sp_h[q].N), (int)q);
+        RC(bt->upload(&g.sp, g.sp_h));
+    }
     if (!g.bnd_h.empty()) RC(bt->upload(&g.bnd, g.bnd_h));
     if (!g.smembers_h.empty()) {
         RC(bt->upload(&g.smembers, g.smembers_h));
@@ -1143,7 +1170,8 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
 
 // The one-warp windows (k_wave) hold a batch of one lattice and one kind of boundary that is small
 // enough to be bound by latency, unless a kernel was asked for.  Bounded FP32 D1Q5 members that
-// k_ring_nee holds stay there: it adds a node's flux differences in another order.
+// stay on k_ring_nee in a large batch (not lbh::span_ok) stay there in a small one: it adds a node's
+// flux differences in another order, and a member's result does not depend on its batch.
 int plan_waves(lbhpde_batch_s *bt, bool *taken) {
     *taken = false;
     Group *g = nullptr;
@@ -1168,7 +1196,8 @@ int plan_waves(lbhpde_batch_s *bt, bool *taken) {
     const bool nee = bt->nbounded > 0;
     std::vector<Seg> m;
     for (int i : g->members) {
-        if (nee && lbh::ring_nee_ok(bt->esz, g->b, bt->segs_h[i])) return LBHPDE_OK;
+        if (nee && lbh::ring_nee_ok(bt->esz, g->b, bt->segs_h[i]) && !lbh::span_ok(bt->esz, g->b, bt->segs_h[i]))
+            return LBHPDE_OK;
         m.push_back(bt->segs_h[i]);
     }
     int dev = 0, sms = 0;
@@ -1454,7 +1483,7 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
     bool any_stream = false, any_res = false;
     for (auto &g : bt->bgroups) {
         if (!g.smembers_h.empty()) any_stream = true;
-        if (!g.bnd_h.empty() || g.rn_h.ncta()) any_res = true;
+        if (!g.bnd_h.empty() || !g.sp_h.empty() || g.rn_h.ncta()) any_res = true;
     }
     int a = cur0;
     if (any_stream) {
@@ -1478,6 +1507,17 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
                                             bt->st[target], bt->coefT, pbd, stride, done, n, bt->stream));
                 ++bt->launches;
                 done += n;
+            }
+            for (size_t q = 0; q < g.sp_first.size(); ++q) {
+                const int i0 = g.sp_first[q].second;
+                const int n = (q + 1 < g.sp_first.size() ? g.sp_first[q + 1].second : (int)g.sp_h.size()) - i0;
+                for (long done = 0; done < nsteps;) {
+                    const int ns = (int)std::min<long>(nsteps - done, 1L << 28);
+                    RC(lbh::launch_span(g.sp_first[q].first, g.sp + i0, n, bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT,
+                                        pbd, stride, done, ns, bt->stream));
+                    ++bt->launches;
+                    done += ns;
+                }
             }
             if (g.bnd_h.empty()) continue;
             for (long done = 0; done < nsteps;) {
