@@ -10,16 +10,16 @@ the device-resident initial profiles (a1), 1000 collide+stream steps (a2-a6) and
 diagnostics reduction (a7).  The model set-up (a0) happens once, at batch creation.
 ``value`` is lattice node-updates per second over all ranks.
 
---workload long_grid: the 2^24-node Kawahara grid (D1Q7, 1000 steps) in temporally blocked
-windows; with --kernel stream, on the one-step-per-launch streaming kernel (HBM roofline).
+--workload long_grid: the 2^24-node Kawahara grid (D1Q7, 1000 steps) in temporally blocked strips
+(FP32) or windows (FP64); with --kernel stream, on the one-step-per-launch streaming kernel (HBM roofline).
 --workload bounded: a tau sweep of Example 4.1 on its bounded grid (non-equilibrium
 extrapolation boundary, A_40 left out as for Table I): --sweep-members instances of N = 601,
 dx = 0.1, dt = 1e-3, tau spread over [1.989, 2.6], 1000 steps, one shared boundary array;
-every instance resident (FP32: 16 nodes a thread, 13 instances a CTA; FP64: one CTA each), 11856
+every instance resident (FP32: a warp each; FP64: a CTA each), 11856
 instances by default (78 per SM).
 --workload nu_grid: a 2^24-node periodic grid of u_t + u^1.5 u_x + u_xxx = 0 (class (1) with a
-real exponent), 1000 steps in on-chip windows (the real-exponent variant evaluates phi^nu once
-per node; ALU roofline), or on the streaming kernel with --kernel stream (HBM roofline).
+real exponent), 1000 steps in temporally blocked strips (the real-exponent variant evaluates phi^nu
+once per node; ALU roofline), or on the streaming kernel with --kernel stream (HBM roofline).
 --impl reference: the CPU oracle timed on the host cores on a bounded sample of the workload.
 """
 from __future__ import annotations
@@ -180,14 +180,14 @@ def workload_problems(args, rank=0, world=1):
         probs, nsteps = [p], p.nsteps
         desc = (f"gkdv_real_exponent_grid: N={args.nodes}, u_t + u^1.5 u_x + u_xxx = 0, D1Q5 scheme 1, "
                 f"dx=0.1, dt=1e-4, tau=1.3, {nsteps} steps per benchmark step ("
-                f"{'streaming kernel' if args.kernel == 'stream' else 'temporally blocked windows'}, "
+                f"{'streaming kernel' if args.kernel == 'stream' else 'temporally blocked on chip'}, "
                 f"phi^nu once per node)")
     else:
         p = W.long_grid_config(N=args.nodes, nsteps=1000)
         probs, nsteps = [p], p.nsteps
         desc = (f"kawahara_long_grid: N={args.nodes}, D1Q7 scheme 1, dx=0.1, dt=1e-4, tau=2.02, "
                 f"{nsteps} steps per benchmark step "
-                f"({'streaming kernel' if args.kernel == 'stream' else 'temporally blocked windows'})")
+                f"({'streaming kernel' if args.kernel == 'stream' else 'temporally blocked on chip'})")
     return probs, nsteps, desc
 
 
@@ -397,9 +397,8 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": ("k_ring_nee<float,5,16,512,5,D2> (13 instances a CTA, interior nodes in registers, "
-                               "depth-2 inflow rebuilt by its reader at fixed register positions)" if esz == 4 else
-                               "k_bounded<double,5,4,512,5> (one resident CTA per instance)"),
+                    "kernel": ("k_span<20> (one warp per instance, its nodes in registers)" if esz == 4 else
+                               "k_bounded<double,5,K,512,5> (one resident CTA per instance, 3 to 6 nodes a thread)"),
                     "flops_per_node_update": fl, "peak_source": src}
         elif args.workload == "nu_grid" and args.kernel != "stream":
             A, Dg = nu_shape(L, probs[0])
@@ -408,7 +407,8 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": f"k_onchip<{'float' if esz == 4 else 'double'},5,K,...,-1> (halo windows, phi^nu)",
+                    "kernel": ("k_strip<5,9,4,1> (strips of one warp, phi^nu)" if esz == 4 else
+                               "k_stream_rt<double,5,256> (run-time degree, phi^nu)"),
                     "flops_per_node_update": fl, "peak_source": src}
         elif args.workload == "nu_grid":
             by = bytes_per_node_update(b, esz)
@@ -423,11 +423,8 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": (f"k_ring<float,5,16,512,5> (every member resident: whole waves at 16 nodes a "
-                               f"thread, then the tail on k_onchip<float,5,8,512,0,5>)"
-                               if args.workload == "ensemble" and esz == 4 else
-                               f"k_onchip<{'float' if esz == 4 else 'double'},{b},K> "
-                               f"({'resident instances + halo windows' if args.workload == 'ensemble' else 'halo windows'})"),
+                    "kernel": (f"k_strip<{b},{D}> (strips of one warp, 16 steps a launch)" if esz == 4 else
+                               f"k_onchip<double,{b},K> (windows that load the SMs evenly)"),
                     "flops_per_node_update": fl, "peak_source": src}
         else:
             by = bytes_per_node_update(b, esz)
@@ -603,11 +600,9 @@ def serving_leg(args, L, torch):
 
 def small_configs_leg(L, torch, stream, refs):
     """Configurations 1 (KdV soliton, N = 400, t = 1, 100 000 steps) and 2 (Kuramoto-Sivashinsky,
-    N = 1024, t = 10, 100 000 steps), each in FP64 and FP32 on the automatic kernel: the whole
-    instance resident in one CTA (one SM) for every step, with as many threads as it has node
-    pairs, since a grid this small has no more parallel work than one CTA holds and more CTAs
-    would need a grid-wide exchange each step (latency-bound: a step is a barrier, an exchange
-    and two nodes' arithmetic per thread).
+    N = 1024, t = 10, 100 000 steps), each in FP64 and FP32 on the automatic kernel: windows of one
+    warp each, spread over the SMs, that trade their borders every few steps (latency-bound: a
+    step is the chain of one node's arithmetic and its share of a trade).
     CUDA-event time of the steps, E and relative L2 against the exact solution (KdV) or the
     ETDRK4 reference (KS), and the oracle's single-thread rate on the host beside it."""
     out = {}
@@ -619,8 +614,7 @@ def small_configs_leg(L, torch, stream, refs):
             else:
                 ref = refs[name]["reference"] if refs and name in refs else W.ks_spectral_reference(t_end=p.t_end)
                 ref_kind = "Fourier ETDRK4 reference"
-            rec = {"N": p.N, "steps": p.nsteps, "dt": p.dt, "tau": p.tau, "error_against": ref_kind,
-                   "ctas": 1, "sms": 1}
+            rec = {"N": p.N, "steps": p.nsteps, "dt": p.dt, "tau": p.tau, "error_against": ref_kind}
             for prec, tag in ((L.FP64, "fp64"), (L.FP32_DEV, "fp32")):
                 sv = L.Solver.for_problem(p, precision=prec)
                 sv.set_phi(p.phi0).step(500)
@@ -638,9 +632,9 @@ def small_configs_leg(L, torch, stream, refs):
                             "node_updates_s": p.N * p.nsteps / sec,
                             "E": float(np.abs(phi - ref).sum() / np.abs(ref).sum()),
                             "l2": float(np.linalg.norm(phi - ref) / np.linalg.norm(ref)),
-                            "kernel": (f"k_onchip<{'float' if tag == 'fp32' else 'double'},5,2,1024,false,5>: the "
-                                       f"whole instance resident in one CTA, 2 nodes a thread (the automatic "
-                                       f"choice for a batch too small to give every SM a warp)")}
+                            "kernel": (f"k_wave<{'float' if tag == 'fp32' else 'double'},5>: one-warp windows spread over "
+                                       f"the SMs (the automatic choice for a batch small enough to be bound "
+                                       f"by latency)")}
             rec["fp32_E_over_fp64_E"] = rec["fp32"]["E"] / rec["fp64"]["E"]
             if refs and name in refs:
                 rec["oracle_single_thread"] = refs[name]["oracle"]
