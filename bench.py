@@ -397,7 +397,7 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": ("k_span<20> (one warp per instance, its nodes in registers)" if esz == 4 else
+                    "kernel": ("k_span<5,20> (one warp per instance, its nodes in registers)" if esz == 4 else
                                "k_bounded<double,5,K,512,5> (one resident CTA per instance, 3 to 6 nodes a thread)"),
                     "flops_per_node_update": fl, "peak_source": src}
         elif args.workload == "nu_grid" and args.kernel != "stream":

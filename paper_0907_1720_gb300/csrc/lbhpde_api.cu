@@ -1081,21 +1081,32 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.bnd_K = K;
     int maxthr = 0, maxD = 0, maxDn = 0;
     bool real = false;
-    // FP32 D1Q5 polynomial members take a warp each where lbh::span_ok says so (automatic choice),
-    // else the 16-node resident kernel (unless a kernel or 4 nodes a thread was asked for), the
+    // FP32 polynomial members take a warp each where lbh::span_ok says so (automatic choice), else
+    // (D1Q5) the 16-node resident kernel (unless a kernel or 4 nodes a thread was asked for), the
     // others one CTA each (real-exponent members on its variant with the generalised f^eq) or the
     // streaming step
     std::vector<lbh::NeeMember> nee;
     const bool nee_auto = bt->kernel == LBHPDE_KERNEL_AUTO || (bt->kernel == LBHPDE_KERNEL_ONCHIP && bt->K_req != K4);
+    // D1Q7 members (k_bounded's otherwise, which gives the same bits) take a warp each from three an
+    // SM on: 304 of 768 nodes 1.26 us a step against 1.04, 250 of 700 1.34 : 1.06, 608 of 601 1.16 : 2.43
+    bool spans = bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0;
+    if (spans && g.b == 7 && bt->esz == 4) {
+        int dev = 0, sms = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const auto n = std::count_if(g.members.begin(), g.members.end(), [&](int i) { return lbh::span_ok(bt->esz, g.b, bt->segs_h[i]); });
+        spans = n > 2 * sms;
+    }
     for (int i : g.members) {
         const Seg &sg = bt->segs_h[i];
-        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && lbh::span_ok(bt->esz, g.b, sg)) {
+        if (spans && lbh::span_ok(bt->esz, g.b, sg)) {
             lbk::SpanInst I{};
             I.off = sg.off;
             I.ld = sg.ld;
             I.N = sg.N;
             I.D = sg.D;
             I.gcoef = sg.coef;
+            I.depth = sg.pad;
             I.mi = i;
             g.sp_h.push_back(I);
             continue;
@@ -1513,7 +1524,7 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
                 const int n = (q + 1 < g.sp_first.size() ? g.sp_first[q + 1].second : (int)g.sp_h.size()) - i0;
                 for (long done = 0; done < nsteps;) {
                     const int ns = (int)std::min<long>(nsteps - done, 1L << 28);
-                    RC(lbh::launch_span(g.sp_first[q].first, g.sp + i0, n, bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT,
+                    RC(lbh::launch_span(g.b, g.sp_first[q].first, g.sp + i0, n, bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT,
                                         pbd, stride, done, ns, bt->stream));
                     ++bt->launches;
                     done += ns;

@@ -210,11 +210,11 @@ double strip_cost(int b, int AA, int DG, int nwarps, int sms);
 int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
                  const void *coefT, int nsteps, cudaStream_t st);
 
-// Bounded FP32 D1Q5 members of one warp each (k_span, lbhpde_span.cu): whether a member can, and the nodes
+// Bounded FP32 members of one warp each (k_span, lbhpde_span.cu): whether a member can, and the nodes
 // a lane holds then (a multiple of 4).
 bool span_ok(size_t esz, int b, const lbk::Seg &s);
 int span_nodes(int N);
-int launch_span(int K, const lbk::SpanInst *insts, int n, const void *in, void *out, const void *coefT, const double *phib,
+int launch_span(int b, int K, const lbk::SpanInst *insts, int n, const void *in, void *out, const void *coefT, const double *phib,
                 long long stride, long long step0, int nsteps, cudaStream_t st);
 
 }  // namespace lbh
