@@ -26,7 +26,9 @@
 //     its own).  Clusters are independent of one another.
 //   grid: boxes in global memory (L2), for instances over as many SMs as they take.  All windows
 //     must be on the GPU together (a cooperative launch).  The trades' numbers run on from launch to
-//     launch in device memory (ctrl[0]), so a captured launch can be replayed.
+//     launch in device memory (ctrl[0]), so a captured launch can be replayed.  A window reads its
+//     first copies from the state that its neighbours overwrite at the end: a fence before its first
+//     trade and one after its last make every such read come before the write.
 // Every wait is bounded: a window whose wait runs out marks ctrl[2], stops waiting and writes NaN,
 // so that every later readout reports it.
 //
@@ -502,8 +504,19 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     };
 
-    // cluster: every box is empty and every first copy read before anybody writes
-    if (csize > 0) cluster_sync();
+    // the lanes' accesses before it come before the lanes' after it, also as other windows see them
+    auto fence = [&] {
+        __syncwarp();
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        __syncwarp();
+    };
+
+    // every first copy is read before anybody writes over it: cluster: (every box is empty, too) by
+    // the barrier; grid: before this window's first trade, which its neighbours await before they write
+    if (csize > 0)
+        cluster_sync();
+    else
+        fence();
     const bool alone = !used || (I.left < 0 && I.right < 0);  // a whole bounded grid: nothing to trade
     int done = 0;
     if (used) {
@@ -521,6 +534,7 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
                 if (!alone) trade();
             }
         }
+        if (csize == 0) fence();  // the neighbours' trades, so their reads, come before these writes
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int p = pos + k;
@@ -536,10 +550,12 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
     }
     if (csize > 0) {
         cluster_sync();  // no CTA ends while a neighbour may still write into its boxes
-    } else if (used && lane == 0) {
-        // the last window to finish moves the trades' numbers on for the next launch
-        __threadfence();
-        if (atomicAdd(ctrl + 1, 1u) == (unsigned)(nused - 1)) {
+    } else if (used) {
+        // the last window to finish moves the trades' numbers on for the next launch, after every
+        // window has read them
+        fence();
+        if (lane == 0 && atomicAdd(ctrl + 1, 1u) == (unsigned)(nused - 1)) {
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
             ctrl[1] = 0;
             ctrl[0] = base + (unsigned)((nsteps - 1) / tblk) + 1u;
         }

@@ -133,3 +133,15 @@ def test_replayed_capture_and_other_streams(L):
         got = s.read_phi()
         s.close()
     assert np.array_equal(got, want) and np.array_equal(got2[0], want2)
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("eq,N", [("kdv", 9001), ("kawahara", 20011)])
+def test_short_calls_in_place(L, eq, N, prec):
+    """Windows over many SMs, back to back calls around the steps between two trades: the copies a
+    window reads at a call's start are what its neighbours overwrite at the call's end."""
+    p = problem(eq, N, 0)
+    calls = [1] * 60 + [2, 3, 5, 9, 17] * 12
+    a, n = solve(L, [p], prec, L.KERNEL_AUTO, calls)
+    b, _ = solve(L, [p], prec, L.KERNEL_STREAM, [sum(calls)])
+    assert n == 1 and np.isfinite(b).all() and np.array_equal(a, b)
