@@ -200,7 +200,7 @@ int lbhpde_step_nee(lbhpde_t h, long nsteps, const double *phib, int phib_on_dev
 /* Step a7: copy phi (t = steps taken * dt) into phi_out ([N] doubles, host or device).
  * Synchronises the stream (host output: the copy; device output: the 4-byte non-finite flag the
  * copy kernel raises).  Returns LBHPDE_ERR_DIVERGED (after copying) if phi has a non-finite
- * value. */
+ * value, LBHPDE_ERR_CUDA if that is because a step's launch failed on the device. */
 int lbhpde_read_phi(lbhpde_t h, double *phi_out, int out_on_device);
 
 /* Diagnostics of step a7, reduced on the GPU in double precision. */
@@ -284,7 +284,8 @@ int lbhpde_batch_step(lbhpde_batch_t b, long nsteps);
  * bounded member.  Periodic members ignore phib. */
 int lbhpde_batch_step_nee(lbhpde_batch_t b, long nsteps, const double *phib, long member_stride,
                           int phib_on_device);
-/* phi_out: [sum N] doubles, host or device.  LBHPDE_ERR_DIVERGED if any phi is non-finite. */
+/* phi_out: [sum N] doubles, host or device.  LBHPDE_ERR_DIVERGED if any phi is non-finite (or
+ * LBHPDE_ERR_CUDA, as lbhpde_read_phi). */
 int lbhpde_batch_read_phi(lbhpde_batch_t b, double *phi_out, int out_on_device);
 /* out: [count] records.  phistar: [sum N] doubles in device memory, or NULL. */
 int lbhpde_batch_diagnostics(lbhpde_batch_t b, const double *phistar_device, lbhpde_diag *out);

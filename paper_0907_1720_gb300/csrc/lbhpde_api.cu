@@ -145,6 +145,7 @@ struct lbhpde_batch_s {
     long long graph_launches[2] = {0, 0};  // kernels in each captured graph
     long steps = 0;
     bool initialised = false;
+    bool wave_failed = false;  // a window of k_wave gave up waiting since the state was set
     std::vector<std::pair<void *, size_t>> allocations;
 
     int dev_alloc(void **p, size_t bytes) {
@@ -1590,6 +1591,22 @@ int batch_step(lbhpde_batch_s *bt, long nsteps, const double *phib = nullptr, lo
     return LBHPDE_OK;
 }
 
+// What a readout that found a non-finite phi returns: LBHPDE_ERR_CUDA where a window of k_wave gave up
+// waiting for a neighbour (it leaves a mark and writes NaN), LBHPDE_ERR_DIVERGED where the solve
+// itself went there.  Only such a readout looks at the mark, and takes it down.
+int nonfinite_cause(lbhpde_batch_s *bt) {
+    for (int gi = 0; gi < 4; ++gi) {
+        Group &g = gi < 2 ? bt->groups[gi] : bt->bgroups[gi - 2];
+        unsigned mark = 0;
+        if (!g.wv_ctrl) continue;
+        CK(cudaMemcpyAsync(&mark, g.wv_ctrl + 2, sizeof mark, cudaMemcpyDeviceToHost, bt->stream));
+        CK(cudaMemsetAsync(g.wv_ctrl + 2, 0, sizeof mark, bt->stream));
+        CK(cudaStreamSynchronize(bt->stream));
+        bt->wave_failed = bt->wave_failed || mark;
+    }
+    return bt->wave_failed ? LBHPDE_ERR_CUDA : LBHPDE_ERR_DIVERGED;
+}
+
 int batch_set_phi(lbhpde_batch_s *bt, const double *phi0, int on_device) {
     lbh::TraceRange trace("lbhpde.set_phi");
     if (!phi0) return LBHPDE_ERR_ARG;
@@ -1608,6 +1625,7 @@ int batch_set_phi(lbhpde_batch_s *bt, const double *phi0, int on_device) {
     }
     bt->steps = 0;
     bt->initialised = true;
+    bt->wave_failed = false;
     return LBHPDE_OK;
 }
 
@@ -1633,7 +1651,7 @@ int batch_read_phi(lbhpde_batch_s *bt, double *out, int on_device) {
         CK(cudaMemcpyAsync(out, bt->phi_buf, sizeof(double) * bt->total, cudaMemcpyDeviceToHost, bt->stream));
     CK(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, bt->stream));
     CK(cudaStreamSynchronize(bt->stream));
-    if (bad) return LBHPDE_ERR_DIVERGED;
+    if (bad) return nonfinite_cause(bt);
     return LBHPDE_OK;
 }
 
@@ -1667,7 +1685,7 @@ int batch_diag(lbhpde_batch_s *bt, const double *phistar, lbhpde_diag *out) {
         d.steps = bt->steps;
         if (h[i].nonfinite) rc = LBHPDE_ERR_DIVERGED;
     }
-    return rc;
+    return rc == LBHPDE_OK ? rc : nonfinite_cause(bt);
 }
 
 int batch_create(lbhpde_batch_s **out, int count, const lbhpde_instance *members, int precision, void *stream,
@@ -1826,6 +1844,7 @@ extern "C" int lbhpde_batch_load(lbhpde_batch_t b, const void *buf, size_t bytes
     b->cur = 0;
     b->steps = (long)h.steps;
     b->initialised = true;
+    b->wave_failed = false;
     return LBHPDE_OK;
 }
 extern "C" int lbhpde_checkpoint_size(lbhpde_t h, size_t *bytes) {

@@ -29,8 +29,9 @@
 //     launch in device memory (ctrl[0]), so a captured launch can be replayed.  A window reads its
 //     first copies from the state that its neighbours overwrite at the end: a fence before its first
 //     trade and one after its last make every such read come before the write.
-// Every wait is bounded: a window whose wait runs out marks ctrl[2], stops waiting and writes NaN,
-// so that every later readout reports it.
+// Every wait is bounded: a window whose wait runs out marks ctrl[2], takes no further step, trades
+// nothing more and writes NaN.  Its neighbours wait for its next trade in vain and do the same, so
+// no value of a solve that a window has left counts as a result, and the readouts report it.
 //
 // The update of a node is that of k_onchip and k_stream (and, at the ends of a bounded grid, of
 // k_bounded and k_nee_fix) operation by operation, so every result is theirs bit for bit.
@@ -55,7 +56,10 @@ struct WaveWin {
 };
 
 constexpr int kWaveWarps = 4;            // windows a CTA: one per scheduler
-constexpr int kWaveWaitLimit = 1 << 22;  // polls of a wait, at most (seconds)
+#ifndef LBK_WAVE_WAIT_LIMIT  // (a test of a wait that runs out compiles the kernel with fewer)
+#define LBK_WAVE_WAIT_LIMIT (1 << 22)
+#endif
+constexpr int kWaveWaitLimit = LBK_WAVE_WAIT_LIMIT;  // polls of a wait, at most (seconds)
 
 // One traded value: 8 bytes in FP32 (value, number), 16 in FP64 (half, number, half, number).
 // Generic addresses: global memory or (distributed) shared memory.  Predicated, not branched: most
@@ -493,10 +497,11 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
 #pragma unroll
                 for (int i = 0; i < JG; ++i) ok &= WaveWord<T>::get(t, rp + ((1 + i) * PITCH + k) * WB, v[i][k], tag);
             }
-            if (dead || __all_sync(0xffffffffu, ok)) break;
+            if (__all_sync(0xffffffffu, ok)) break;
             if (tries >= kWaveWaitLimit) {
                 dead = true;  // uniform: the vote and the count are
                 if (lane == 0) atomicExch(ctrl + 2, 1u);
+                break;
             }
         }
     };
@@ -524,7 +529,7 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
         // grid: the state is updated in place, so nobody may write before its neighbours have read
         // their first copies: at least one trade comes before
         if (csize == 0 && nsteps <= tblk && !alone) trade();
-        while (done < nsteps) {
+        while (done < nsteps && !dead) {
             const int n = min(tblk, nsteps - done);
             ends_ready();
             for (int s = 0; s < n; ++s) step(s);
@@ -534,6 +539,7 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
                 if (!alone) trade();
             }
         }
+        ends_ready();  // (a window that gave up has copies under way)
         if (csize == 0) fence();  // the neighbours' trades, so their reads, come before these writes
 #pragma unroll
         for (int k = 0; k < K; ++k) {

@@ -145,3 +145,22 @@ def test_short_calls_in_place(L, eq, N, prec):
     a, n = solve(L, [p], prec, L.KERNEL_AUTO, calls)
     b, _ = solve(L, [p], prec, L.KERNEL_STREAM, [sum(calls)])
     assert n == 1 and np.isfinite(b).all() and np.array_equal(a, b)
+
+
+def test_wait_that_runs_out(L, tmp_path):
+    """A window that gives up waiting leaves a mark and NaN, and so do all that depend on it
+    (tests/wave_giveup.cu, the kernel with few polls a wait)."""
+    import os
+    import subprocess
+    from paper_0907_1720_gb300 import build as B
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    libdir, exe = os.path.dirname(B.build()), str(tmp_path / "wave_giveup")
+    nvcc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc")
+    cmd = [nvcc, "-std=c++17", "-O2", "-gencode", "arch=compute_103a,code=sm_103a", "-DLBK_WAVE_WAIT_LIMIT=4096",
+           "-I", os.path.join(root, "include"), "-I", os.path.join(root, "paper_0907_1720_gb300", "csrc"),
+           os.path.join(root, "tests", "wave_giveup.cu"), "-o", exe, "-L", libdir, "-llbhpde", "-lcudart",
+           "-Xlinker", "-rpath=" + libdir]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert out.returncode == 0 and out.stdout.startswith("ok"), out.stdout[-2000:]
