@@ -1070,14 +1070,18 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.sblocks_h.clear();
     int K = lbh::kBoundedK;
     const int K4 = K;
-    if (bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && !g.has_nu && lbh::onchip_dc(g.b, g.maxD) > 0) {
-        std::vector<Seg> m;
+    if (bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && !g.has_nu) {
+        std::vector<Seg> m;  // what k_bounded will hold: their degree says which of its variants runs
+        int D = 0;
         for (int i : g.members)
-            if (bt->N[i] <= (long long)K * lbh::kBoundedMaxT) m.push_back(bt->segs_h[i]);
+            if (bt->N[i] <= (long long)K * lbh::kBoundedMaxT) {
+                m.push_back(bt->segs_h[i]);
+                D = std::max(D, bt->segs_h[i].D);
+            }
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (!m.empty() && sms > 0) K = lbh::bounded_nodes(g.b, m, sms);
+        if (lbh::onchip_dc(g.b, D) == lbh::bounded_degree(g.b) && sms > 0) K = lbh::bounded_nodes(g.b, m, sms);
     }
     g.bnd_K = K;
     int maxthr = 0, maxD = 0, maxDn = 0;

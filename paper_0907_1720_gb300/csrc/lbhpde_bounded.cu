@@ -45,7 +45,7 @@ int launch_bounded_t(const BoundedArgs &a) {
 
 template <typename T, int B>
 int launch_bounded_d(int dc, const BoundedArgs &a) {
-    constexpr int DC = B == 5 ? 5 : 7;
+    constexpr int DC = bounded_degree(B);
     if constexpr (sizeof(T) == 8) {  // FP64: the nodes a thread of the plan
         if (dc == DC && a.K == 3) return launch_bounded_t<T, B, DC, 3, kBoundedMaxTAny>(a);
         if (dc == DC && a.K == 5) return launch_bounded_t<T, B, DC, 5, kBoundedMaxTAny>(a);

@@ -142,3 +142,27 @@ def test_fp64_bounded_nodes_a_thread(L, example, count, N, depth):
         out.append(b.read_phi())
         b.close()
     assert np.isfinite(out[2]).all() and np.array_equal(out[0], out[2]) and np.array_equal(out[1], out[2])
+
+
+LINEAR = W.Equation("linear", (1.0, 0.0, 0.1), ((0.0, 1.0), (), (0.0, 1.0)))  # degree 1
+
+
+@pytest.mark.parametrize("make", [lambda i: (W.mkdv(), 601), lambda i: (W.mkdv() if i % 5 == 0 else W.kdv(), 601),
+                                  lambda i: (W.gks_cubic(), 301), lambda i: (W.kdv(), 3001) if i == 7 else (LINEAR, 601)],
+                         ids=["cubic", "cubic and quadratic", "degree above 9", "long quadratic, short linear"])
+def test_fp64_bounded_other_degrees(L, make):
+    """FP64 bounded members whose degree k_bounded has not compiled (all of them, one in five, or the
+    short ones beside a longer member of the compiled degree, which streams): as the streaming step."""
+    ps = []
+    for i in range(304):
+        eq, N = make(i)
+        phi0 = 0.3 + 0.2 * np.cos(2 * np.pi * (np.arange(N) / N + 0.01 * i))
+        ps.append(W.Problem(eq, N, 0.1, 1e-5, 1.1 + 0.001 * i, 0, phi0, boundary="nee", meta={"depth": 2}))
+    pb = 0.4 + 0.01 * np.random.default_rng(5).random((40, 4))
+    out = []
+    for kernel in (L.KERNEL_AUTO, L.KERNEL_STREAM):
+        b = L.Batch(ps, precision=L.FP64).set_kernel(kernel)
+        b.set_phi(np.concatenate([p.phi0 for p in ps])).step_nee(1, pb[:1]).step_nee(39, np.ascontiguousarray(pb[1:]))
+        out.append(b.read_phi())
+        b.close()
+    assert np.isfinite(out[1]).all() and np.array_equal(out[0], out[1])
