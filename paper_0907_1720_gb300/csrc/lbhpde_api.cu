@@ -1321,8 +1321,10 @@ int choose_kernels(lbhpde_batch_s *bt) {
     return LBHPDE_OK;
 }
 
-// nsteps steps of the periodic members (groups); bt->cur ends on the buffer that holds them.
-int step_periodic(lbhpde_batch_s *bt, long nsteps) {
+// nsteps steps of the periodic members (groups); bt->cur ends on the buffer that holds them.  *back: the
+// caller has to copy that buffer to the one the call began in, once the bounded members are in it too.
+int step_periodic(lbhpde_batch_s *bt, long nsteps, bool *back) {
+    *back = false;
     bool any_stream = false, any_halo = false;
     for (auto &g : bt->groups) {
         if (g.members.empty()) continue;
@@ -1452,10 +1454,7 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps) {
         for (int c = 0; c < lbh::kRingClasses; ++c)
             if (used[c]) CK(cudaStreamWaitEvent(bt->stream, bt->ev_join[c], 0));
     bt->cur = cur1;
-    if (captured && cur1 != cur0) {
-        CK(cudaMemcpyAsync(bt->st[cur0], bt->st[cur1], bt->st_bytes, cudaMemcpyDeviceToDevice, bt->stream));
-        bt->cur = cur0;
-    }
+    *back = captured && cur1 != cur0;
     return LBHPDE_OK;
 }
 
@@ -1589,8 +1588,13 @@ int batch_step(lbhpde_batch_s *bt, long nsteps, const double *phib = nullptr, lo
     bool any_periodic = false;
     for (auto &g : bt->groups)
         if (!g.members.empty()) any_periodic = true;
-    if (any_periodic) RC(step_periodic(bt, nsteps));
+    bool back = false;
+    if (any_periodic) RC(step_periodic(bt, nsteps, &back));
     if (bt->nbounded) RC(step_bounded(bt, nsteps, pbd, stride, cur0, any_periodic));
+    if (back) {  // (the bounded members have read the buffer that this writes)
+        CK(cudaMemcpyAsync(bt->st[cur0], bt->st[bt->cur], bt->st_bytes, cudaMemcpyDeviceToDevice, bt->stream));
+        bt->cur = cur0;
+    }
     bt->steps += nsteps;
     return LBHPDE_OK;
 }

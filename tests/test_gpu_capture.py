@@ -1,0 +1,77 @@
+"""Captured calls, replayed: a call has to end in the buffer it began in, whatever kernels a batch's
+members take and however many launches the call is.  Each against the streaming kernel's steps
+launched one by one, equal bit for bit."""
+import numpy as np
+import pytest
+
+from paper_0907_1720_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0907_1720_gb300 import build as B
+    B.build()
+    from paper_0907_1720_gb300 import lbhpde
+    lbhpde.lib()
+    return lbhpde
+
+
+def periodic(N, i=0):
+    phi0 = 0.4 + 0.3 * np.cos(2 * np.pi * (np.arange(N) / N + 0.1 * i))
+    return W.Problem(W.kdv(), int(N), 0.1, 1e-5, 1.1, 0, phi0)
+
+
+def bounded(N):
+    xl = -0.05 * (N - 1)
+    return W.Problem(W.ks(), N, 0.1, 1e-3, 1.989, 0, W.ks_shock(W.grid(xl, N, 0.1), 0.0), xl=xl, scheme=1 | 0x100, boundary="nee",
+                     exact_xt=W.ks_shock, meta={"depth": 2})
+
+
+BATCHES = {  # (precision, members): windows or strips, residents, each beside bounded ones
+    "fp32 strips, one bounded warp": (1, lambda: [periodic(N, i) for i, N in enumerate([4000, 700, 9001] * 150)] + [bounded(601)] * 3),
+    "fp32 windows and residents": (1, lambda: [periodic(20000), periodic(300, 1)] + [bounded(601)]),
+    "fp64 windows": (0, lambda: [periodic(N, i) for i, N in enumerate([200003, 300])] + [bounded(601)] * 3),
+    "fp64 windows, streamed bounded": (0, lambda: [periodic(100003), bounded(3001), bounded(301)]),
+}
+
+
+def replayed(L, ps, prec, kernel, steps, phib, replays=3):
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        b = L.Batch(ps, precision=prec).set_kernel(*kernel)
+        b.set_phi(np.concatenate([p.phi0 for p in ps]))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            b.step(steps) if phib is None else b.step_nee(steps, phib)
+        for _ in range(replays):
+            g.replay()
+        got = b.read_phi()
+        b.close()
+    return got
+
+
+def streamed(L, ps, prec, steps, phib, calls=3):
+    b = L.Batch(ps, precision=prec).set_kernel(L.KERNEL_STREAM)
+    b.set_phi(np.concatenate([p.phi0 for p in ps]))
+    for _ in range(calls):
+        b.step(steps) if phib is None else b.step_nee(steps, phib)
+    out = b.read_phi()
+    b.close()
+    return out
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 17])
+@pytest.mark.parametrize("name", list(BATCHES))
+def test_mixed_batches(L, name, steps):
+    prec, make = BATCHES[name]
+    ps = make()
+    phib = torch.from_numpy(W.boundary_values(bounded(601), 2, 0, steps)).cuda()
+    got = replayed(L, ps, prec, (L.KERNEL_AUTO,), steps, phib)
+    want = streamed(L, ps, prec, steps, phib)
+    assert np.isfinite(want).all() and np.array_equal(got, want)
