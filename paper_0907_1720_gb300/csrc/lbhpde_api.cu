@@ -1390,11 +1390,11 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps, bool *back) {
         if (!g.members.empty() && g.windows()) tb = std::min(tb, g.tblk);
     long nchunks = any_halo ? (nsteps + tb - 1) / tb : 0;
     // a captured call is replayed with the buffers it was captured with: it has to end in the one it
-    // began in (an even number of launches, or a copy back after a single step)
+    // began in (an even number of launches of a step or more each, or a copy back)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool captured = (nchunks & 1) && bt->stream != nullptr && cudaStreamIsCapturing(bt->stream, &cap) == cudaSuccess &&
                           cap != cudaStreamCaptureStatusNone;
-    if (captured && nsteps > 1) ++nchunks;
+    if (captured && nchunks < nsteps) ++nchunks;
     const int cur0 = bt->cur, cur1 = bt->cur ^ (int)(nchunks & 1);
     // resident instances (each size class) and windows touch disjoint rows: when there is more
     // than one kind, they run concurrently, the resident classes on streams of their own

@@ -75,3 +75,27 @@ def test_mixed_batches(L, name, steps):
     got = replayed(L, ps, prec, (L.KERNEL_AUTO,), steps, phib)
     want = streamed(L, ps, prec, steps, phib)
     assert np.isfinite(want).all() and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 7])
+@pytest.mark.parametrize("prec,K", [(0, 4), (1, 8)], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("per_launch", [1, 2])
+def test_windows_of_few_steps_a_launch(L, per_launch, prec, K, steps):
+    """Windows of one or two steps a launch (asked for), with residents beside them."""
+    ps = [periodic(20011), periodic(300, 1), periodic(5000, 2)]
+    got = replayed(L, ps, prec, (L.KERNEL_ONCHIP, K, per_launch), steps, None)
+    want = streamed(L, ps, prec, steps, None)
+    assert np.isfinite(want).all() and np.array_equal(got, want)
+
+
+def test_tuned_one_step_a_launch(L):
+    """The same from a tuned pair of one step a launch (a degree that nothing else here uses)."""
+    eq = W.Equation("linear", (1.0, 0.0, 0.1), ((0.0, 1.0), (), (0.0, 1.0)))
+    ps = [W.Problem(eq, 9001 + 11 * i, 0.1, 1e-5, 1.1, 0, periodic(9001 + 11 * i).phi0) for i in range(2)]
+    want = streamed(L, ps, 0, 3, None)
+    L.set_tuning(L.FP64, 5, 1, 4, 1)
+    try:
+        got = replayed(L, ps, 0, (L.KERNEL_HALO,), 3, None)
+    finally:
+        L.set_tuning(L.FP64, 5, 1, 4, 64)  # the untuned pair, for the tests that follow
+    assert np.isfinite(want).all() and np.array_equal(got, want)
