@@ -467,7 +467,7 @@ int pack_ring(int b, size_t esz, int K, int dc, const std::vector<Member> &m, Pa
     } else {
         out.smem = (size_t(4) * ne * out.nthreads + size_t(2) * ne * out.max_inst + coef_max) * esz;
     }
-    if (out.smem > 227 * 1024) return LBHPDE_ERR_UNSUPPORTED;
+    if (out.smem > kMaxSmem) return LBHPDE_ERR_UNSUPPORTED;
     return LBHPDE_OK;
 }
 

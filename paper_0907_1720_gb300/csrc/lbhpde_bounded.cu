@@ -36,7 +36,7 @@ struct BoundedArgs {
 template <typename T, int B, int DC, int K = kBoundedK, int MAXT = kBoundedMaxT>
 int launch_bounded_t(const BoundedArgs &a) {
     auto fn = lbk::k_bounded<T, B, K, MAXT, DC>;
-    LBB_CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem));
+    if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
     fn<<<a.ninst, a.nthreads, a.smem, a.st>>>((const T *)a.in, (T *)a.out, a.insts, (const T *)a.coefT, a.phib,
                                              a.stride, a.step0, a.nsteps);
     LBB_CK(cudaGetLastError());

@@ -30,6 +30,18 @@ struct TraceRange {
 constexpr int kChunk = 1024;          // nodes per block of the node-parallel kernels
 constexpr int kGenericThreads = 256;  // init / readout / diagnostics threads per block
 
+// The dynamic shared memory a CTA can have (none of the kernels that take any has static one too), and
+// a kernel's permission to use it all, whatever a launch takes.  The permission belongs to the kernel
+// in the whole process: with each launch asking for its own size, a smaller plan of another handle's
+// thread could take it down between a launch's asking and the launch, which then failed.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <typename F>
+bool allow_smem(F fn) {
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
+}
+
 // One instance to place on the on-chip kernel.
 struct Member {
     lbk::Seg seg;      // placement of the current state (and its coefficient block)

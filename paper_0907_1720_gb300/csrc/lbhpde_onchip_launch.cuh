@@ -37,7 +37,7 @@ struct OnchipArgs {
 template <typename T, int B, int K, int MAXT, bool HALO, int DC>
 int launch_onchip_t(const OnchipArgs &a) {
     auto fn = lbk::k_onchip<T, B, K, MAXT, HALO, DC>;
-    LBH_OCK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.p->smem));
+    if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
     fn<<<a.p->ncta(), a.p->nthreads, a.p->smem, a.st>>>((const T *)a.in, (T *)a.out, a.insts, a.first,
                                                          (const T *)a.coefT, a.nsteps, a.p->max_inst);
     LBH_OCK(cudaGetLastError());

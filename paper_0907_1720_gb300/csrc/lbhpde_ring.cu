@@ -17,10 +17,7 @@ template <int MAXT, int DC>
 int launch_ring_t(const Packed &p, const lbk::OnchipInst *insts, const int *first, const void *in, void *out,
                   const void *coefT, int nsteps, cudaStream_t st) {
     auto fn = lbk::k_ring<float, 5, kRingK, MAXT, DC>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return LBHPDE_ERR_CUDA;
-    }
+    if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
     fn<<<p.ncta(), p.nthreads, p.smem, st>>>((const float *)in, (float *)out, insts, first, (const float *)coefT,
                                              nsteps);
     if (cudaGetLastError() != cudaSuccess) return LBHPDE_ERR_CUDA;
@@ -55,10 +52,7 @@ int launch_ring_nee_t(const PackedNee &p, const lbk::RingNeeInst *insts, const i
                       const void *coefT, const double *phib, long long stride, long long step0, int nsteps,
                       cudaStream_t st) {
     auto fn = lbk::k_ring_nee<float, 5, kRingK, MAXT, DC, D2>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return LBHPDE_ERR_CUDA;
-    }
+    if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
     fn<<<p.ncta(), p.nthreads, p.smem, st>>>((const float *)in, (float *)out, insts, first, (const float *)coefT, phib,
                                              stride, step0, nsteps);
     if (cudaGetLastError() != cudaSuccess) return LBHPDE_ERR_CUDA;
@@ -152,7 +146,7 @@ int pack_ring_nee(int b, int dc, const std::vector<NeeMember> &m, PackedNee &out
     out.nthreads = (out.nthreads + 31) & ~31;
     out.stride = threads;
     out.smem = (size_t(lbk::nee_fixed_elems(b, threads)) + coef_max) * sizeof(float);
-    if (out.smem > 227 * 1024) return LBHPDE_ERR_UNSUPPORTED;
+    if (out.smem > kMaxSmem) return LBHPDE_ERR_UNSUPPORTED;
     return LBHPDE_OK;
 }
 

@@ -89,10 +89,7 @@ int launch_strip_t(const PackedStrip &p, const lbk::StripSeg *segs, const int *f
                    const void *coefT, int nsteps, cudaStream_t st) {
     auto fn = lbk::k_strip<B, DC, AA, DG>;
     const int smem = lbk::strip_smem(B, AA, DC);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return LBHPDE_ERR_CUDA;
-    }
+    if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
     fn<<<p.nwarps(), 32, smem, st>>>((const float *)in, (float *)out, segs, first, p.nmix(), (const float *)coefT, nsteps);
     if (cudaGetLastError() != cudaSuccess) return LBHPDE_ERR_CUDA;
     return LBHPDE_OK;

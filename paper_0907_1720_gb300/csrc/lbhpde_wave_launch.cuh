@@ -31,7 +31,7 @@ template <typename T, int B, int K, int G, int DC, bool NEE>
 int launch_wave_t(const WaveArgs &a) {
     auto fn = lbk::k_wave<T, B, K, G, DC, NEE>;
     const PackedWave &p = *a.p;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess ||
+    if (!allow_smem(fn) ||
         (p.csize > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         (void)cudaGetLastError();
         return LBHPDE_ERR_CUDA;
@@ -377,7 +377,7 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
         const size_t boxes = (size_t)lbk::wave_box_bytes((int)esz, b, k.K, k.G);
         out.smem = (size_t(out.wsmem) * esz + (k.C > 0 ? boxes : 0)) * lbk::kWaveWarps;
         out.box_bytes = k.C > 0 ? 0 : boxes * out.wins.size();
-        if (out.smem > 227 * 1024) continue;
+        if (out.smem > kMaxSmem) continue;
         int room = 0;
         WaveArgs a{};
         a.p = &out;
