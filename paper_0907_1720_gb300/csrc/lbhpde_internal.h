@@ -196,6 +196,8 @@ struct PackedWave {
 bool pack_wave(const std::vector<lbk::Seg> &m, int b, int K, int G, int T, int csize, std::vector<lbk::WaveWin> &out);
 // The plan of a whole batch, where k_wave is the better kernel for it on a GPU of `sms` SMs.
 bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms, PackedWave &out);
+// What a step of its best form costs on that GPU by the model, in SM clocks (as cta_cost, strip_cost).
+double wave_cost(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms);
 // nsteps steps, in place; ends: the table of launch_wave_ends for the same steps (bounded members).
 int launch_wave(const PackedWave &p, const lbk::WaveWin *wins, unsigned char *box, unsigned *ctrl, void *st, const void *coefT,
                 int nsteps, const void *ends, cudaStream_t stream);

@@ -308,21 +308,20 @@ double strip_cost(int b, int AA, int DG, int nwarps, int sms) {
     return two + (full - 1) * more + (rest == 0 ? 0.0 : (rest <= 0.5 ? 0.54 * more : more));
 }
 
-bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms, PackedWave &out) {
-    out = PackedWave{};
+namespace {
+
+// The forms, depths and placements of k_wave for a batch, and the modelled cost of a step of each.
+std::vector<WavePick> wave_picks(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms) {
     const int W = lbk::wmax(b);
-    long long total = 0;
     int D = 0;
     bool real = false, fixed = true;
     for (const lbk::Seg &x : m) {
-        total += x.N;
         D = std::max(D, x.D);
         real = real || x.A > 0;
         if (x.A > 0 && !lbk::wave_fixed_rows(b, x.A, x.Dg)) fixed = false;
     }
-    if (total > (1 << 19)) return false;  // the other kernels fill the GPU
-    const int DC = b == 5 ? 5 : 7;
-    const double ops = wave_ops(b, dc > 0 ? DC : D), scale = real ? 1.0 : ops / wave_ops(b, DC);
+    // (the forms' costs are those of degree 5 on D1Q5, 7 on D1Q7)
+    const double scale = real ? 1.0 : wave_ops(b, dc > 0 ? dc : D) / wave_ops(b, b == 5 ? 5 : 7);
     std::vector<WavePick> picks;
     for (const WaveForm &f : kWaveForms) {
         if (f.esz != (int)esz || f.b != b) continue;
@@ -352,6 +351,29 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
                 picks.push_back(WavePick{f.K, f.G, T, C, q * (f.a * scale + extra) + X / T});
             }
     }
+    return picks;
+}
+
+}  // namespace
+
+double wave_cost(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms) {
+    double least = HUGE_VAL;
+    for (const WavePick &k : wave_picks(esz, b, dc, nee, m, sms)) least = std::min(least, k.cost);
+    return least;
+}
+
+bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> &m, int sms, PackedWave &out) {
+    out = PackedWave{};
+    long long total = 0;
+    int D = 0;
+    bool real = false;
+    for (const lbk::Seg &x : m) {
+        total += x.N;
+        D = std::max(D, x.D);
+        real = real || x.A > 0;
+    }
+    if (total > (1 << 19)) return false;  // the other kernels fill the GPU
+    std::vector<WavePick> picks = wave_picks(esz, b, dc, nee, m, sms);
     std::stable_sort(picks.begin(), picks.end(), [](const WavePick &x, const WavePick &y) { return x.cost < y.cost; });
     double other = cta_cost(esz, b, dc, nee, real, m, sms);
     int AA = 0, DG = 0;

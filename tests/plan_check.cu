@@ -1,0 +1,38 @@
+// Host-side check of the estimates that choose the kernels (no GPU): they follow the degree.  Prints
+// "ok" and exits 0, or the first violation and exits 1.
+#include <cstdio>
+#include <vector>
+
+#include "lbhpde_internal.h"
+
+static int fails = 0;
+#define CHECK(c, ...)                                        \
+    do {                                                     \
+        if (!(c) && fails++ == 0) {                          \
+            std::printf("FAIL %s:%d: ", __FILE__, __LINE__); \
+            std::printf(__VA_ARGS__);                        \
+            std::printf("\n");                               \
+        }                                                    \
+    } while (0)
+
+static std::vector<lbk::Seg> members(int count, int N, int D) {
+    lbk::Seg s{};
+    s.N = N;
+    s.D = D;
+    return std::vector<lbk::Seg>(count, s);
+}
+
+int main() {
+    const int sms = 152;
+    // a cubic flux (degree 9 of D1Q5) takes 4 (9 + 3) + 1 operations a node where a quadratic one takes
+    // 4 (5 + 3) + 1: FP64, where those are the cost of a step, in k_wave's estimate as in the others'
+    for (int count : {16, 64, 128}) {
+        const auto m5 = members(count, 1000, 5), m9 = members(count, 1000, 9);
+        const double w5 = lbh::wave_cost(8, 5, 5, false, m5, sms), w9 = lbh::wave_cost(8, 5, 9, false, m9, sms);
+        const double c5 = lbh::cta_cost(8, 5, 5, false, false, m5, sms), c9 = lbh::cta_cost(8, 5, 9, false, false, m9, sms);
+        CHECK(w9 > 1.3 * w5 && w9 < 1.49 * w5, "%d members: k_wave %g and %g", count, w5, w9);
+        CHECK(c9 > 1.3 * c5 && c9 < 1.49 * c5, "%d members: CTAs %g and %g", count, c5, c9);
+    }
+    if (!fails) std::printf("ok\n");
+    return fails ? 1 : 0;
+}
