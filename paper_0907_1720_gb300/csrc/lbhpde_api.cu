@@ -26,6 +26,7 @@ namespace {
 
 constexpr int kStreamThreads = kChunk / 4;  // k_stream: one group of 4 nodes per thread
 constexpr int kGraphSteps = 64;             // one-step launches per captured graph (even)
+constexpr int kSides = 6;                   // side streams of a batch, at most
 
 #define CK(call)                                              \
     do {                                                      \
@@ -104,10 +105,25 @@ struct lbhpde_batch_s {
     size_t esz = 8;
     int count = 0;
     cudaStream_t stream = nullptr;
-    // resident instances run on `side`, forked from and joined back into `stream` with events,
-    // so that the window launches fill the SMs the resident launch leaves idle
-    cudaStream_t side[lbh::kRingClasses] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join[lbh::kRingClasses] = {};
+    // launches of disjoint members run on `side`, forked from and joined back into `stream` with
+    // events, so that one fills the SMs another leaves idle
+    cudaStream_t side[kSides] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
+    // side stream i, waiting for what `stream` held at the fork (ev_fork has been recorded)
+    int fork_side(int i, cudaStream_t *st) {
+        if (!side[i]) {
+            CK(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
+            CK(cudaEventCreateWithFlags(&ev_join[i], cudaEventDisableTiming));
+        }
+        CK(cudaStreamWaitEvent(side[i], ev_fork, 0));
+        *st = side[i];
+        return LBHPDE_OK;
+    }
+    int record_fork() {
+        if (!ev_fork) CK(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
+        CK(cudaEventRecord(ev_fork, stream));
+        return LBHPDE_OK;
+    }
     // streaming path: kGraphSteps one-step launches captured once per buffer parity and replayed
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool has_alloc = false;
@@ -199,7 +215,7 @@ struct lbhpde_batch_s {
         for (auto &gx : graph)
             if (gx) cudaGraphExecDestroy(gx);
         graph[0] = graph[1] = nullptr;
-        for (int c = 0; c < lbh::kRingClasses; ++c) {
+        for (int c = 0; c < kSides; ++c) {
             if (side[c]) cudaStreamDestroy(side[c]);
             if (ev_join[c]) cudaEventDestroy(ev_join[c]);
             side[c] = nullptr;
@@ -1068,8 +1084,10 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     g.sp_first.clear();
     g.smembers_h.clear();
     g.sblocks_h.clear();
-    int K = lbh::kBoundedK;
+    int K = lbh::kBoundedK, dev = 0, sms = 0;
     const int K4 = K;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && !g.has_nu) {
         std::vector<Seg> m;  // what k_bounded will hold: their degree says which of its variants runs
         int D = 0;
@@ -1078,10 +1096,7 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
                 m.push_back(bt->segs_h[i]);
                 D = std::max(D, bt->segs_h[i].D);
             }
-        int dev = 0, sms = 0;
-        CK(cudaGetDevice(&dev));
-        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (lbh::onchip_dc(g.b, D) == lbh::bounded_degree(g.b) && sms > 0) K = lbh::bounded_nodes(g.b, m, sms);
+        if (lbh::onchip_dc(g.b, D) == lbh::bounded_degree(g.b)) K = lbh::bounded_nodes(g.b, m, sms);
     }
     g.bnd_K = K;
     int maxthr = 0, maxD = 0, maxDn = 0;
@@ -1096,9 +1111,6 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     // SM on: 304 of 768 nodes 1.26 us a step against 1.04, 250 of 700 1.34 : 1.06, 608 of 601 1.16 : 2.43
     bool spans = bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0;
     if (spans && g.b == 7 && bt->esz == 4) {
-        int dev = 0, sms = 0;
-        CK(cudaGetDevice(&dev));
-        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const auto n = std::count_if(g.members.begin(), g.members.end(), [&](int i) { return lbh::span_ok(bt->esz, g.b, bt->segs_h[i]); });
         spans = n > 2 * sms;
     }
@@ -1171,9 +1183,9 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
     if (!g.sp_h.empty()) {
         std::stable_sort(g.sp_h.begin(), g.sp_h.end(),
                          [](const lbk::SpanInst &x, const lbk::SpanInst &y) { return lbh::span_nodes(x.N) > lbh::span_nodes(y.N); });
-        for (size_t q = 0; q < g.sp_h.size(); ++q)  // a launch for each number of nodes a lane
-            if (q == 0 || lbh::span_nodes(g.sp_h[q].N) != g.sp_first.back().first)
-                g.sp_first.emplace_back(lbh::span_nodes(g.sp_h[q].N), (int)q);
+        std::vector<int> nodes;
+        for (const lbk::SpanInst &I : g.sp_h) nodes.push_back(lbh::span_nodes(I.N));
+        g.sp_first = lbh::span_launches(nodes, sms);
         RC(bt->upload(&g.sp, g.sp_h));
     }
     if (!g.bnd_h.empty()) RC(bt->upload(&g.bnd, g.bnd_h));
@@ -1409,21 +1421,11 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps, bool *back) {
         kinds += used[c] ? 1 : 0;
     }
     const bool fork = kinds > 1;
-    if (fork) {
-        if (!bt->ev_fork) CK(cudaEventCreateWithFlags(&bt->ev_fork, cudaEventDisableTiming));
-        CK(cudaEventRecord(bt->ev_fork, bt->stream));
-    }
+    if (fork) RC(bt->record_fork());
     for (int c = 0; c < lbh::kRingClasses; ++c) {
         if (!used[c]) continue;
         cudaStream_t rs = bt->stream;
-        if (fork) {
-            if (!bt->side[c]) {
-                CK(cudaStreamCreateWithFlags(&bt->side[c], cudaStreamNonBlocking));
-                CK(cudaEventCreateWithFlags(&bt->ev_join[c], cudaEventDisableTiming));
-            }
-            CK(cudaStreamWaitEvent(bt->side[c], bt->ev_fork, 0));
-            rs = bt->side[c];
-        }
+        if (fork) RC(bt->fork_side(c, &rs));
         for (auto &g : bt->groups) {
             if (g.members.empty() || (g.waves && c == 0)) continue;
             const bool tail = g.waves && c == lbh::kRingClasses - 1 && g.ring[0].ncta();
@@ -1515,36 +1517,70 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
     }
     const int target = fixed ? bt->cur : (any_stream ? a : cur0);
     if (any_res) {
+        // The launches of the resident members, each of all steps: the ones that take longest first.
+        enum { kRingNee, kBounded, kSpan };
+        struct Kind {
+            Group *g;
+            int what, K, first, count;  // kSpan: nodes a lane, and of the group's members in that order
+        };
+        std::vector<Kind> kinds;
         for (auto &g : bt->bgroups) {
-            for (long done = 0; g.rn_h.ncta() && done < nsteps;) {
-                const int n = (int)std::min<long>(nsteps - done, 1L << 30);
-                RC(lbh::launch_ring_nee_f32(g.rn_dc, g.rn_h, g.rn_insts, g.rn_first, bt->st[done == 0 ? cur0 : target],
-                                            bt->st[target], bt->coefT, pbd, stride, done, n, bt->stream));
-                ++bt->launches;
-                done += n;
-            }
+            if (g.rn_h.ncta()) kinds.push_back(Kind{&g, kRingNee, 0, 0, 0});
+            if (!g.bnd_h.empty()) kinds.push_back(Kind{&g, kBounded, 0, 0, 0});
+        }
+        for (auto &g : bt->bgroups)
             for (size_t q = 0; q < g.sp_first.size(); ++q) {
                 const int i0 = g.sp_first[q].second;
                 const int n = (q + 1 < g.sp_first.size() ? g.sp_first[q + 1].second : (int)g.sp_h.size()) - i0;
-                for (long done = 0; done < nsteps;) {
-                    const int ns = (int)std::min<long>(nsteps - done, 1L << 28);
-                    RC(lbh::launch_span(g.b, g.sp_first[q].first, g.sp + i0, n, bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT,
-                                        pbd, stride, done, ns, bt->stream));
-                    ++bt->launches;
-                    done += ns;
-                }
+                kinds.push_back(Kind{&g, kSpan, g.sp_first[q].first, i0, n});
             }
-            if (g.bnd_h.empty()) continue;
+        // side by side: each takes as long as its slowest member, whether or not it fills the GPU (GB300,
+        // us a call of 1 and of 48 steps, side by side and one after another: 248 FP32 members of 364 to
+        // 1459 nodes 50, 140 and 79, 359; 6 of 327 to 1309 20, 65 and 41, 211)
+        const bool fork = kinds.size() > 1;
+        if (fork) RC(bt->record_fork());
+        bool used[kSides] = {};
+        auto launch = [&](size_t i) -> int {
+            Group &g = *kinds[i].g;
+            cudaStream_t st = bt->stream;
+            const int sd = (int)((i + kSides - 1) % kSides);  // (the first on the batch's own stream)
+            if (fork && i > 0) {
+                if (used[sd])
+                    st = bt->side[sd];
+                else
+                    RC(bt->fork_side(sd, &st));
+                used[sd] = true;
+            }
             for (long done = 0; done < nsteps;) {
-                const int n = (int)std::min<long>(nsteps - done, lbh::bounded_launch_steps(g.b, bt->esz));
-                const size_t smem = lbh::bounded_smem(g.b, bt->esz, g.bnd_threads, g.bnd_D, n);
-                RC(lbh::launch_bounded(g.b, bt->esz, g.bnd_dc, (int)g.bnd_h.size(), g.bnd_threads, smem, g.bnd,
-                                       bt->st[done == 0 ? cur0 : target], bt->st[target], bt->coefT, pbd, stride,
-                                       done, n, bt->stream, g.bnd_K));
+                const void *in = bt->st[done == 0 ? cur0 : target];
+                void *out = bt->st[target];
+                int n;
+                if (kinds[i].what == kRingNee) {
+                    n = (int)std::min<long>(nsteps - done, 1L << 30);
+                    RC(lbh::launch_ring_nee_f32(g.rn_dc, g.rn_h, g.rn_insts, g.rn_first, in, out, bt->coefT, pbd, stride, done, n, st));
+                } else if (kinds[i].what == kSpan) {
+                    n = (int)std::min<long>(nsteps - done, 1L << 28);
+                    RC(lbh::launch_span(g.b, kinds[i].K, g.sp + kinds[i].first, kinds[i].count, in, out,
+                                        bt->coefT, pbd, stride, done, n, st));
+                } else {
+                    n = (int)std::min<long>(nsteps - done, lbh::bounded_launch_steps(g.b, bt->esz));
+                    const size_t smem = lbh::bounded_smem(g.b, bt->esz, g.bnd_threads, g.bnd_D, n);
+                    RC(lbh::launch_bounded(g.b, bt->esz, g.bnd_dc, (int)g.bnd_h.size(), g.bnd_threads, smem, g.bnd, in, out, bt->coefT,
+                                           pbd, stride, done, n, st, g.bnd_K));
+                }
                 ++bt->launches;
                 done += n;
             }
-        }
+            return LBHPDE_OK;
+        };
+        int rc = LBHPDE_OK;
+        for (size_t i = 0; i < kinds.size() && rc == LBHPDE_OK; ++i) rc = launch(i);
+        for (int i = 0; i < kSides; ++i)  // (also after a failure: what was launched belongs to the stream)
+            if (used[i]) {
+                CK(cudaEventRecord(bt->ev_join[i], bt->side[i]));
+                CK(cudaStreamWaitEvent(bt->stream, bt->ev_join[i], 0));
+            }
+        RC(rc);
     }
     if (any_stream && a != target) {
         for (auto &g : bt->bgroups)

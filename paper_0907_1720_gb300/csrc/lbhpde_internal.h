@@ -230,6 +230,9 @@ int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *fir
 // a lane holds then (a multiple of 4).
 bool span_ok(size_t esz, int b, const lbk::Seg &s);
 int span_nodes(int N);
+// The launches of members sorted by their own nodes a lane, falling: (nodes a lane, first member) of
+// at most two; a member may run with more than its own.
+std::vector<std::pair<int, int>> span_launches(const std::vector<int> &nodes, int sms);
 int launch_span(int b, int K, const lbk::SpanInst *insts, int n, const void *in, void *out, const void *coefT, const double *phib,
                 long long stride, long long step0, int nsteps, cudaStream_t st);
 

@@ -1,6 +1,8 @@
 // Launch of k_span (bounded FP32 instances of one warp each).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "lbhpde.h"
 #include "lbhpde_internal.h"
 #include "lbhpde_span.cuh"
@@ -19,6 +21,30 @@ bool span_ok(size_t esz, int b, const lbk::Seg &s) {
     const bool form = b == 5 ? s.D <= 5 && s.pad == 2 && s.N >= 96 && s.N <= 1024
                              : s.D <= 7 && (s.pad == 1 || s.pad == 2) && s.N > 128 && s.N <= 768;
     return esz == 4 && s.A == 0 && form && 5 * s.N >= 3 * 32 * span_nodes(s.N);
+}
+
+// Not one for each number of nodes a lane: the code of one is tens of KB, and an SM that runs four or
+// more of them side by side waits for instructions (GB300, us a step: 250 members of 1000 nodes 0.87,
+// and 250 of 500 beside them 0.95, but 250 of each of 1000, 880, 700 and 500 3.1, as long as one after
+// another).  Two side by side take the sum of what each takes of the schedulers, a warp alone on one
+// at least its own time: with the largest number of nodes for all, or with a second one, whichever is
+// less by this (us a step on D1Q5, which measured, of 608, 1000, 2000 and 4000 members: 32 nodes a
+// lane 1.07, 1.63, 3.06, 5.2; 16 nodes 0.71, 0.97, 1.73, 2.77; 8 nodes 0.52, 0.64, 1.07, 1.72).
+std::vector<std::pair<int, int>> span_launches(const std::vector<int> &nodes, int sms) {
+    std::vector<std::pair<int, int>> out;
+    if (nodes.empty()) return out;
+    auto load = [&](int K, size_t n) { return (0.104 + 0.0209 * K) * (double)((n + 4 * sms - 1) / (4 * sms)); };
+    const double alone = 0.42 + 0.0195 * nodes[0];
+    double best = 0.95 * std::max(alone, load(nodes[0], nodes.size()));
+    size_t at = 0;
+    for (size_t q = 1; q < nodes.size(); ++q) {
+        if (nodes[q] == nodes[q - 1]) continue;
+        const double t = std::max(alone, load(nodes[0], q) + load(nodes[q], nodes.size() - q));
+        if (t < best) best = t, at = q;
+    }
+    out.emplace_back(nodes[0], 0);
+    if (at > 0) out.emplace_back(nodes[at], (int)at);
+    return out;
 }
 
 namespace {

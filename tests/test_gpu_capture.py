@@ -99,3 +99,18 @@ def test_tuned_one_step_a_launch(L):
     finally:
         L.set_tuning(L.FP64, 5, 1, 4, 64)  # the untuned pair, for the tests that follow
     assert np.isfinite(want).all() and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("steps", [1, 7, 8, 40])
+def test_unequal_bounded_members(L, steps):
+    """Bounded members whose launches run side by side, captured and not."""
+    ps = [bounded(N) for N in (97, 150, 231, 301, 420, 601, 700, 850, 1000, 601)] * 20  # one warp each, every number of nodes a lane
+    phib = torch.from_numpy(W.boundary_values(bounded(601), 2, 0, steps)).cuda()
+    want = streamed(L, ps, 1, steps, phib)
+    got = replayed(L, ps, 1, (L.KERNEL_AUTO,), steps, phib)
+    b = L.Batch(ps, precision=1)
+    b.set_phi(np.concatenate([p.phi0 for p in ps]))
+    for _ in range(3):
+        b.step_nee(steps, phib)
+    assert np.isfinite(want).all() and np.array_equal(got, want) and np.array_equal(b.read_phi(), want)
+    b.close()

@@ -1,0 +1,70 @@
+"""The automatic choice of kernels against the on-chip kernel asked for (one CTA a member, or windows),
+on batches of unequal members and of several kinds, which are planned kind by kind: it is not the
+slower one.  The allowance of a fifth is for noise: what these batches lost was more."""
+import numpy as np
+import pytest
+
+from paper_0907_1720_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0907_1720_gb300 import build as B
+    B.build()
+    from paper_0907_1720_gb300 import lbhpde
+    lbhpde.lib()
+    return lbhpde
+
+
+EQS = {"kdv": (W.kdv, 1e-5, 1.1), "mkdv": (W.mkdv, 1e-5, 1.2), "kawahara": (W.kawahara, 1e-4, 2.02)}
+ENDS = {"ks": (W.ks, W.ks_shock, 1e-3, 1.989, 1 | 0x100, 2), "kawahara": (W.kawahara, W.kawahara_soliton, 1e-4, 2.02, 1, 1)}
+
+
+def periodic(eq, N):
+    make, dt, tau = EQS[eq]
+    return W.Problem(make(), int(N), 0.1, dt, tau, 0, 0.4 + 0.3 * np.cos(2 * np.pi * np.arange(N) / N))
+
+
+def bounded(eq, N):
+    make, ex, dt, tau, scheme, depth = ENDS[eq]
+    xl = -0.05 * (N - 1)
+    return W.Problem(make(), int(N), 0.1, dt, tau, 0, ex(W.grid(xl, int(N), 0.1), 0.0), xl=xl, scheme=scheme, boundary="nee",
+                     exact_xt=ex, meta={"depth": depth})
+
+
+def spread(count, lo, hi):
+    return np.linspace(lo, hi, count).astype(int).tolist()
+
+
+def us_a_step(L, ps, prec, kernel, phib, steps=48):
+    with torch.cuda.stream(torch.cuda.Stream()):
+        b = L.Batch(ps, precision=prec).set_kernel(kernel)
+        b.set_phi(np.concatenate([p.phi0 for p in ps]))
+        best = 1e30
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            b.step(steps) if phib is None else b.step_nee(steps, phib)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1) * 1e3 / steps)
+        b.close()
+    return best
+
+
+BOUNDED = {"ks, few": ("ks", spread(6, 327, 1309)), "ks, over 1024": ("ks", spread(248, 364, 1459)), "ks, short": ("ks", spread(304, 239, 959)),
+           "ks, many": ("ks", spread(2000, 160, 1000)), "kawahara": ("kawahara", spread(661, 135, 541))}
+
+
+@pytest.mark.parametrize("name", list(BOUNDED))
+def test_unequal_bounded_members(L, name):
+    eq, sizes = BOUNDED[name]
+    ps = [bounded(eq, N) for N in sizes]
+    phib = torch.from_numpy(W.boundary_values(ps[0], 2 if eq == "ks" else 3, 0, 48)).cuda()
+    auto, asked = (us_a_step(L, ps, L.FP32_DEV, k, phib) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
+    assert auto < 1.2 * asked, (auto, asked)
