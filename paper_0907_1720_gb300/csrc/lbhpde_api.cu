@@ -1158,6 +1158,10 @@ int plan_bounded(lbhpde_batch_s *bt, Group &g) {
             for (long long x = 0; x < bt->N[i]; x += kChunk) g.sblocks_h.push_back(make_int2(i, (int)x));
         }
     }
+    // the longest first: CTAs start in this order, and the last ones should be short (GB300, FP64, us a step,
+    // in order of size and in any order: D1Q5, 504 members of 150 to 601 nodes 15.6 and 19.9, 160 of 300 to
+    // 1200 11.9 and 16.0; D1Q7, 504 of 75 to 301 17.4 and 24.0)
+    std::stable_sort(g.bnd_h.begin(), g.bnd_h.end(), [](const lbk::BoundedInst &x, const lbk::BoundedInst &y) { return x.N > y.N; });
     g.bnd_threads = (maxthr + 31) / 32 * 32;
     g.bnd_dc = real ? -1 : lbh::onchip_dc(g.b, maxD);
     g.bnd_D = g.bnd_dc > 0 ? g.bnd_dc : maxD;

@@ -74,27 +74,40 @@ int bounded_shift(int b, int N, int depth, int K) {
     return -1;
 }
 
-// The scheduler with the most warps paces an SM (an FP64 operation of a warp holds it for 64 clocks),
-// and a warp that is half empty costs as much as a full one: of the warps of the ceil(n / SMs)
-// instances of an SM it holds a quarter, rounded up.  601 nodes on D1Q7, two instances an SM (GB300, us a
-// step): 5 warps each at K = 4 21.5, 4 at K = 5 20.8; one instance 12.7 and 11.5; 301 nodes, two, 3 warps at
-// K = 4 13.1, 2 at K = 5 11.6.
+// An SM does the FP64 work of four warps at a time, a warp's alone takes as long as a quarter of four
+// warps' (its own operations one after another), and a warp that is half empty costs as much as a full
+// one.  So a step of the members an SM holds at once takes, in units of one position a lane, K times a
+// quarter of their warps, at least K, and a little more where a quarter is no whole number, on top of a
+// barrier and the ends.  How many it holds the registers say (and every CTA has the warps of the
+// largest member); the rest follow in further rounds.  GB300, us a step at K = 4, 3, 5, 6: D1Q7, 304 of
+// 601 nodes 21.7, 22.9, 20.9, 24.9; 304 of 301 13.3, 12.8, 11.7, 13.8; 160 of 847 (K = 5 and 6: one at a time)
+// 29.3, -, 32.6, 37.5; 1500 of 150 to 601 78.0, 85.2, 82.9, 84.1; D1Q5, 152 of 301 5.35, 4.38, 6.49, 7.56.
 int bounded_nodes(int b, const std::vector<lbk::Seg> &m, int sms) {
     int best = kBoundedK;
     double least = 0;
     for (int K : {kBoundedK, 3, 5, 6}) {
         if (K < lbk::wmax(b)) continue;
+        // warps an SM holds (registers a thread: 128 at K = 4, 154 (D1Q5) and 192 at 3, 214 to 254 at 5 and 6)
+        const int room = K == 4 ? 16 : (K == 3 && b == 5 ? 12 : 8);
         long long warps = 0;
+        int wmost = 1;
         bool fits = true;
         for (const lbk::Seg &s : m) {
             const int shift = bounded_shift(b, s.N, s.pad, K);
             fits = fits && shift >= 0;
-            warps += (s.N + shift + 32 * K - 1) / (32 * K);
+            const int w = (s.N + shift + 32 * K - 1) / (32 * K);
+            warps += w;
+            wmost = std::max(wmost, w);
         }
         if (!fits) continue;
-        const long long ctas = ((long long)m.size() + sms - 1) / sms;  // instances of the fullest SM
-        const double per = (double)warps / m.size() * ctas;
-        const double c = std::ceil(per / 4.0 - 1e-9) * K;
+        const int per_sm = (int)(((long long)m.size() + sms - 1) / sms);  // members of the fullest SM
+        const int at_once = std::min(per_sm, std::max(1, room / wmost));
+        const double mean = per_sm == 1 ? wmost : (double)warps / m.size();
+        auto round = [&](int n) {
+            const double q = n * mean / 4.0;
+            return (b == 5 ? 1.03 : 0.65) + K * std::max(1.0, q + 0.29 * (std::ceil(q - 1e-9) - q));
+        };
+        const double c = per_sm / at_once * round(at_once) + (per_sm % at_once ? round(per_sm % at_once) : 0.0);
         if (least == 0 || c < 0.97 * least) {
             least = c;
             best = K;

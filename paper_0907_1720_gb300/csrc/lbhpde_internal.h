@@ -143,8 +143,7 @@ int bounded_launch_steps(int b, size_t esz);
 int bounded_shift(int b, int N, int depth, int K = kBoundedK);
 // The degree k_bounded has compiled; 3, 5 and 6 nodes a thread exist in FP64 for it alone.
 constexpr int bounded_degree(int b) { return b == 5 ? 5 : 7; }
-// Nodes a thread (4, or 3, 5, 6) with which FP64 bounded members of that degree load the SMs'
-// schedulers most evenly.
+// Nodes a thread (4, or 3, 5, 6) with which FP64 bounded members of that degree take the least time.
 int bounded_nodes(int b, const std::vector<lbk::Seg> &m, int sms);
 // dc: the compiled degree (5 on D1Q5, 7 on D1Q7), 0 for a run-time degree, -1 for the variant
 // that also evaluates real-exponent instances (A > 0).

@@ -1,5 +1,6 @@
-// Host-side check of the estimates that choose the kernels (no GPU): they follow the degree.  Prints
+// Host-side check of the estimates that choose the kernels (no GPU).  Prints
 // "ok" and exits 0, or the first violation and exits 1.
+#include <algorithm>
 #include <cstdio>
 #include <vector>
 
@@ -32,6 +33,20 @@ int main() {
         const double c5 = lbh::cta_cost(8, 5, 5, false, false, m5, sms), c9 = lbh::cta_cost(8, 5, 9, false, false, m9, sms);
         CHECK(w9 > 1.3 * w5 && w9 < 1.49 * w5, "%d members: k_wave %g and %g", count, w5, w9);
         CHECK(c9 > 1.3 * c5 && c9 < 1.49 * c5, "%d members: CTAs %g and %g", count, c5, c9);
+    }
+    // bounded FP64 members on k_bounded: the nodes a thread that measured least (within 3%) on a GPU of 152 SMs
+    const struct {
+        int b, count, lo, hi, K;
+    } bounded[] = {{7, 304, 601, 601, 5}, {7, 304, 301, 301, 5}, {7, 152, 301, 301, 3}, {5, 152, 601, 601, 5}, {5, 304, 847, 847, 4},
+                   {7, 304, 847, 847, 4}, {7, 152, 250, 1000, 4}, {5, 1500, 150, 601, 4}, {7, 504, 450, 450, 4}, {7, 304, 300, 1200, 4}};
+    for (const auto &c : bounded) {
+        std::vector<lbk::Seg> m = members(c.count, c.hi, c.b);
+        for (int i = 0; i < c.count; ++i) {
+            m[i].N = c.lo + (int)((long long)(c.hi - c.lo) * i / std::max(1, c.count - 1));
+            m[i].pad = c.b == 5 ? 2 : 1;
+        }
+        const int K = lbh::bounded_nodes(c.b, m, sms);
+        CHECK(K == c.K, "D1Q%d, %d members of %d to %d nodes: %d nodes a thread", c.b, c.count, c.lo, c.hi, K);
     }
     if (!fails) std::printf("ok\n");
     return fails ? 1 : 0;
