@@ -1399,25 +1399,35 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps, bool *back) {
         for (; left > 0; --left) RC(one_step());
         return LBHPDE_OK;
     }
-    // halo windows advance tblk steps per launch through the ping-pong buffers; ring instances
-    // read the current buffer once and write the buffer the halo launches end in
-    int tb = 1 << 30;
-    for (auto &g : bt->groups)
-        if (!g.members.empty() && g.windows()) tb = std::min(tb, g.tblk);
-    long nchunks = any_halo ? (nsteps + tb - 1) / tb : 0;
-    // a captured call is replayed with the buffers it was captured with: it has to end in the one it
-    // began in (an even number of launches of a step or more each, or a copy back)
+    // windows advance tblk steps per launch through the ping-pong buffers, each group by its own; resident
+    // instances read the current buffer once and write the buffer the windows end in
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool captured = (nchunks & 1) && bt->stream != nullptr && cudaStreamIsCapturing(bt->stream, &cap) == cudaSuccess &&
+    const bool captured = any_halo && bt->stream != nullptr && cudaStreamIsCapturing(bt->stream, &cap) == cudaSuccess &&
                           cap != cudaStreamCaptureStatusNone;
-    if (captured && nchunks < nsteps) ++nchunks;
-    const int cur0 = bt->cur, cur1 = bt->cur ^ (int)(nchunks & 1);
+    long nchunks[2] = {}, most = 0;
+    int odd = 0, even = 0, fixed = 0;  // groups by the parity of their launches; that cannot have one more
+    for (int gi = 0; gi < 2; ++gi) {
+        Group &g = bt->groups[gi];
+        if (g.members.empty() || !g.windows()) continue;
+        nchunks[gi] = (nsteps + g.tblk - 1) / g.tblk;
+        (nchunks[gi] & 1 ? odd : even) += 1;
+        fixed += nchunks[gi] == nsteps;
+    }
+    // All groups end in one buffer.  A captured call is replayed with the buffers it was captured with: it
+    // has to end in the one it began in (an even number of launches, or a copy back where every launch
+    // of an odd number is a step).
+    const int par = fixed ? (int)(nsteps & 1) : (captured || even ? 0 : odd > 0);
+    for (long &n : nchunks) {
+        if (n > 0 && (n & 1) != par) ++n;
+        most = std::max(most, n);
+    }
+    const int cur0 = bt->cur, cur1 = bt->cur ^ par;
     // resident instances (each size class) and windows touch disjoint rows: when there is more
     // than one kind, they run concurrently, the resident classes on streams of their own
     // (a group planned in whole waves launches its tail (class 0) after its full CTAs (class 2), on
     // the same stream)
     bool used[lbh::kRingClasses] = {};
-    int kinds = any_halo ? 1 : 0;
+    int kinds = odd + even;
     for (int c = 0; c < lbh::kRingClasses; ++c) {
         for (auto &g : bt->groups)
             if (!g.members.empty() && (g.ring[c].ncta() || (c == lbh::kRingClasses - 1 && g.waves && g.ring[0].ncta())))
@@ -1447,14 +1457,22 @@ int step_periodic(lbhpde_batch_s *bt, long nsteps, bool *back) {
         }
         if (fork) CK(cudaEventRecord(bt->ev_join[c], bt->side[c]));
     }
-    long left = nsteps;
-    for (long c = 0; c < nchunks; ++c) {
-        const int n = (int)((left + nchunks - c - 1) / (nchunks - c));  // equal parts, at most tb
-        for (auto &g : bt->groups)
-            if (!g.members.empty() && g.windows())
-                RC(launch_group(bt, g, true, bt->st[bt->cur], bt->st[bt->cur ^ 1], n, bt->stream));
-        bt->cur ^= 1;
-        left -= n;
+    // the windows of two groups side by side too, the second one's on a stream of its own: one after
+    // another, a step took the sum of what each group was planned for
+    const bool both = nchunks[0] > 0 && nchunks[1] > 0;
+    cudaStream_t ws[2] = {bt->stream, bt->stream};
+    if (both) RC(bt->fork_side(lbh::kRingClasses, &ws[1]));
+    long left[2] = {nsteps, nsteps};
+    for (long c = 0; c < most; ++c)
+        for (int gi = 0; gi < 2; ++gi) {
+            if (c >= nchunks[gi]) continue;
+            const int n = (int)((left[gi] + nchunks[gi] - c - 1) / (nchunks[gi] - c));  // equal parts, at most tblk
+            RC(launch_group(bt, bt->groups[gi], true, bt->st[cur0 ^ (c & 1)], bt->st[cur0 ^ (c & 1) ^ 1], n, ws[gi]));
+            left[gi] -= n;
+        }
+    if (both) {
+        CK(cudaEventRecord(bt->ev_join[lbh::kRingClasses], ws[1]));
+        CK(cudaStreamWaitEvent(bt->stream, bt->ev_join[lbh::kRingClasses], 0));
     }
     if (fork)
         for (int c = 0; c < lbh::kRingClasses; ++c)

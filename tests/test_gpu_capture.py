@@ -114,3 +114,31 @@ def test_unequal_bounded_members(L, steps):
         b.step_nee(steps, phib)
     assert np.isfinite(want).all() and np.array_equal(got, want) and np.array_equal(b.read_phi(), want)
     b.close()
+
+
+def kawahara(N):
+    return W.Problem(W.kawahara(), int(N), 0.1, 1e-4, 2.02, 0, 0.4 + 0.3 * np.cos(2 * np.pi * np.arange(N) / N))
+
+
+LATTICES = {  # two groups with windows or strips of depths of their own, residents beside them
+    "fp64 windows": (0, (0, 0, 0), lambda: [periodic(200003), periodic(300, 1), kawahara(100003), kawahara(500)]),
+    "fp32 strips": (1, (0, 0, 0), lambda: [periodic(700001), kawahara(600001)]),
+    "fp32 strips and windows": (1, (0, 0, 0), lambda: [periodic(700001), kawahara(20011), kawahara(300)]),
+    "one step a launch": (0, (3, 4, 1), lambda: [periodic(9001), kawahara(5003)]),
+}
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 17, 40])
+@pytest.mark.parametrize("name", list(LATTICES))
+def test_two_lattices(L, name, steps):
+    """The windows of the two lattices run side by side and end in one buffer, captured or not."""
+    prec, kernel, make = LATTICES[name]
+    ps = make()
+    want = streamed(L, ps, prec, steps, None)
+    assert np.isfinite(want).all() and np.array_equal(replayed(L, ps, prec, kernel, steps, None), want)
+    b = L.Batch(ps, precision=prec).set_kernel(*kernel)
+    b.set_phi(np.concatenate([p.phi0 for p in ps]))
+    for _ in range(3):
+        b.step(steps)
+    assert np.array_equal(b.read_phi(), want)
+    b.close()

@@ -1,6 +1,6 @@
 """The automatic choice of kernels against the on-chip kernel asked for (one CTA a member, or windows),
 on batches of unequal members and of several kinds, which are planned kind by kind: it is not the
-slower one.  The allowance of a fifth is for noise: what these batches lost was more."""
+slower one.  The allowances (FP32 times are short) are for noise: what these batches lost was more."""
 import numpy as np
 import pytest
 
@@ -68,3 +68,16 @@ def test_unequal_bounded_members(L, name):
     phib = torch.from_numpy(W.boundary_values(ps[0], 2 if eq == "ks" else 3, 0, 48)).cuda()
     auto, asked = (us_a_step(L, ps, L.FP32_DEV, k, phib) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
     assert auto < 1.2 * asked, (auto, asked)
+
+
+LATTICES = {"cubic, few": (0, [("mkdv", 294)] * 10 + [("kawahara", N) for N in (55711, 222846)]),
+            "cubic, long": (0, [("mkdv", 1500)] * 2 + [("kawahara", N) for N in spread(28, 4050, 16200)]),
+            "quadratic": (0, [("kdv", N) for N in spread(3, 113, 453)] + [("kawahara", 207784)] * 2)}
+
+
+@pytest.mark.parametrize("name", list(LATTICES))
+def test_two_lattices(L, name):
+    prec, members = LATTICES[name]
+    ps = [periodic(*m) for m in members]
+    auto, asked = (us_a_step(L, ps, prec, k, None) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
+    assert auto < 1.06 * asked, (auto, asked)
