@@ -218,9 +218,9 @@ struct PackedStrip {
 bool strip_ok(size_t esz, int b, int dc, const std::vector<lbk::Seg> &m, int *AA, int *DG);
 void pack_strip(int b, int AA, int DG, const std::vector<lbk::Seg> &m, PackedStrip &out);
 // What a step costs on a GPU of `sms` SMs, in SM clocks: the CTA-wide kernels on a group's members,
-// k_strip with that many warps.
+// k_strip with a plan.
 double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms);
-double strip_cost(int b, int AA, int DG, int nwarps, int sms);
+double strip_cost(const PackedStrip &p, int sms);
 // At most lbk::strip_steps(b, AA) steps, from buffer `in` to another one.
 int launch_strip(const PackedStrip &p, const lbk::StripSeg *segs, const int *first, const void *in, void *out,
                  const void *coefT, int nsteps, cudaStream_t st);

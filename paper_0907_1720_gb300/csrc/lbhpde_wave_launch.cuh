@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <functional>
 
 #include "lbhpde.h"
 #include "lbhpde_internal.h"
@@ -250,13 +251,59 @@ long long wave_windows(const lbk::Seg &s, int W, int cap, int T) {
 
 }  // namespace
 
+namespace {
+
+// A step of k_ring on the members it holds (FP32 D1Q5), in SM clocks, by the plan it gets (GB300).  Whole
+// waves and a tail: 3400 a wave.  CTAs by size class, four of 128 threads an SM, two of 256 or one of 512:
+// by the warps of the fullest SM's schedulers, one to four [107 members of 1095 nodes, a CTA on an SM,
+// 1600; 249 of 1635, two, 1760; 318 CTAs of 960 nodes, three, 2540; 565 of 1287, four, 2740; 85 of 4021
+// in CTAs of 256 threads 2050, 231 of 2710 2290; 107 of 4184 in CTAs of 512 2600, 81 of 6638 3260].  A
+// warp takes the writes past its members' ends once for each remainder of 16 [1318 members of 43 to 173
+// nodes 3930, 431 of 133 to 534 2600, 303 of 455 to 1821 2080; equal members of any size 1600 to 1700].
+double ring_cost(const std::vector<lbk::Seg> &m, int sms) {
+    std::vector<Member> res, full, tail, cls[kRingClasses];
+    long long nodes = 0;
+    bool equal = true;
+    for (const lbk::Seg &s : m)
+        if (s.N <= 512 * kRingK) {
+            res.push_back(Member{s, 0, 1});
+            nodes += s.N;
+            equal = equal && s.N % kRingK == res[0].seg.N % kRingK;
+        }
+    if (res.empty()) return 0;
+    if (split_ring_waves(5, kRingK, sms, res, full, tail)) {
+        const double waves = nodes / (512.0 * kRingK * sms), rest = waves - std::floor(waves);
+        return 3400 * (std::floor(waves) + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0)));
+    }
+    split_ring_classes(4, 5, kRingK, res, cls);
+    std::vector<int> load(sms, 0);  // warps, the largest CTAs first, each to the emptiest SM (a heap)
+    for (int c = kRingClasses - 1; c >= 0; --c) {
+        Packed p;
+        if (cls[c].empty() || pack_ring(5, 4, kRingK, 5, cls[c], p, ring_class_threads(4, 5, kRingK, c)) != LBHPDE_OK) continue;
+        long long thr = 0;
+        for (const lbk::OnchipInst &I : p.insts) thr += I.nthr;
+        const int warps = (int)((thr + 32LL * p.ncta() - 1) / (32LL * p.ncta()));
+        for (int i = 0; i < p.ncta(); ++i) {
+            std::pop_heap(load.begin(), load.end(), std::greater<int>());
+            load.back() += warps;
+            std::push_heap(load.begin(), load.end(), std::greater<int>());
+        }
+    }
+    const int most = *std::max_element(load.begin(), load.end());
+    const double part[5] = {0, 1650, 1950, 2600, 3300};
+    const double ends = equal ? 0.0 : (150 + 480 * 512.0 * res.size() / nodes) * std::max(1, most / 16);
+    // (what does not fit at once starts as the first CTAs end [612 CTAs of 128 threads 4360, 369 of 256 4490])
+    return most / 16 * part[4] + (most > 16 ? 0.65 : 1.0) * part[(most % 16 + 3) / 4] + ends;
+}
+
+}  // namespace
+
 // The step of the CTA-wide kernels on a group's members, in SM clocks (GB300; measured in brackets).
 //   A CTA alone: a barrier and an exchange, then its nodes at the rate of one SM (KdV on 400 nodes
 //   [580 FP32, 8080 FP64], 2048-node FP64 windows [36 200]).
-//   FP32 windows: D1Q5 900 and then 5.2e11 node-updates/s [600 000 nodes 2430, 2^21 6390], D1Q7 1840 a
-//   wave of 152 windows [400 000 nodes 3620, 10^6 7060].
-//   FP32 D1Q5 residents of a group that fills the GPU (k_ring): 3400 a wave of 152 CTAs of 8192 nodes
-//   [ensemble of 128 members 3430, 400 6730, 4096 47 500].
+//   FP32 windows: D1Q5 650 and then 7.2e11 node-updates/s (real exponents: 450, 6.3e11 of their operations) [616 000 nodes 2470, 10^6 3670, 1.32 10^6 4310,
+//   2^21 6390], D1Q7 1840 a wave of 152 windows [400 000 nodes 3620, 10^6 7060].
+//   FP32 D1Q5 residents of a group that fills the GPU: ring_cost; windows beside them overlap.
 //   Bounded: 601 nodes FP64 [16 400 D1Q5, 29 800 D1Q7], FP32 D1Q7 [2400]; streamed, two launches a
 //   step: FP64 [55 000, 84 900], FP32 [23 400, 29 700].
 double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vector<lbk::Seg> &m, int sms) {
@@ -286,21 +333,27 @@ double cta_cost(size_t esz, int b, int dc, bool nee, bool real, const std::vecto
     }
     double all = (resident + windows) * ops / (rate * sms);
     if (esz == 4 && !nee) {
-        const double waves = resident / (512.0 * kRingK * sms), rest = waves - (long long)waves;
         // (a degree k_ring has not compiled takes single multiply-adds)
-        const double wave = 3400 * ops / wave_ops(5, 5) * (dc == 5 ? 1.0 : 1.5);
-        const double res = ring ? wave * ((long long)waves + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0))) : resident * ops / (60.0 * sms);
-        const double win = windows == 0 ? 0 : (b == 5 ? 450 + windows * ops / (66.0 * sms) : 1840 * std::ceil(windows / (1856.0 * sms)) * ops / wave_ops(7, 7));
-        all = res + win;
+        const double res = ring ? ring_cost(m, sms) * ops / wave_ops(5, 5) * (dc == 5 ? 1.0 : 1.5) : resident * ops / (60.0 * sms);
+        const double win = windows == 0 ? 0 : (b == 5 ? (real ? 450 + windows * ops / (66.0 * sms) : 650 + windows * ops / (75.0 * sms)) : 1840 * std::ceil(windows / (1856.0 * sms)) * ops / wave_ops(7, 7));
+        all = ring ? std::max({res, win, res > 0 && win > 0 ? 0.6 * res + 0.9 * win : 0.0}) : res + win;
+        if (ring) worst = 0;  // (ring_cost has it)
     }
     return std::max(worst, all);
 }
 
 // A step of k_strip: one warp on a scheduler, two, and every further wave of two (GB300: D1Q5 400 000
-// nodes 2160, 800 000 3440, 2^24 37 800; D1Q7 400 000 2840, 800 000 4800, 2^24 75 400).
-double strip_cost(int b, int AA, int DG, int nwarps, int sms) {
+// nodes 2200, 800 000 3500, 2^24 37 800; D1Q7 400 000 2840, 800 000 4800, 2^24 75 400), and more where
+// warps hold several segments or move nodes singly (D1Q5, warps of one or two equal members 2200, of three
+// or of unequal ones 2470, of four 2730).
+double strip_cost(const PackedStrip &p, int sms) {
+    const int b = p.b, AA = p.AA, DG = p.DG, nwarps = p.nwarps();
+    bool unequal = false;
+    for (const lbk::StripSeg &S : p.segs) unequal = unequal || (S.N - p.segs[0].N) % 4 != 0;
+    const double held = p.nmix() ? (double)(p.segs.size() - p.nfull) / p.nmix() : 0.0;  // segments of a mixed warp
+    const double mix = b == 5 ? 270 * std::max({held - 2, unequal ? 1.0 : 0.0, 0.0}) : 0.0;
     const double s = AA > 0 ? (DG == 1 ? 2.0 : 4.9) : wave_ops(b, DG) / wave_ops(b, b == 5 ? 5 : 7);  // the power and the rows (2^24 nodes: 76 000 and 180 000)
-    const double one = s * (b == 5 ? 2100 : 2840), two = s * (b == 5 ? 3440 : 4800), more = s * (b == 5 ? 2570 : 3620);
+    const double one = AA > 0 ? s * 2100 : (b == 5 ? s * (2200 + mix) : s * 2840), two = AA > 0 ? s * 3440 : (b == 5 ? s * (3480 + 0.4 * mix) : s * 4800), more = s * (b == 5 ? 2570 : 3620);
     const double waves = nwarps / (8.0 * sms);
     if (waves <= 0.5) return one;
     if (waves <= 1.0) return two;
@@ -380,7 +433,7 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
     if (!nee && strip_ok(esz, b, dc, m, &AA, &DG)) {
         PackedStrip p;
         pack_strip(b, AA, DG, m, p);
-        other = std::min(other, strip_cost(b, AA, DG, p.nwarps(), sms));
+        other = std::min(other, strip_cost(p, sms));
     }
     for (const WavePick &k : picks) {
         if (k.cost > 0.85 * other) return false;

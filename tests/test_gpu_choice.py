@@ -81,3 +81,16 @@ def test_two_lattices(L, name):
     ps = [periodic(*m) for m in members]
     auto, asked = (us_a_step(L, ps, prec, k, None) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
     assert auto < 1.06 * asked, (auto, asked)
+
+
+STRIPS = {"equal, short": [("kdv", 221)] * 2007, "equal": [("kdv", 960)] * 635, "unequal": [("kdv", N) for N in spread(675, 389, 1558)],
+          "few and long": [("kdv", 410891)] * 2, "over a wave": [("kdv", 630335)] * 2,
+          "two lattices": [("kdv", 4096)] * 100 + [("kawahara", 2048)] * 50}
+
+
+@pytest.mark.parametrize("name", list(STRIPS))
+def test_fp32_members_about_a_wave(L, name):
+    """Strips, windows or residents for FP32 D1Q5 members that about fill the GPU."""
+    ps = [periodic(*m) for m in STRIPS[name]]
+    auto, asked = (us_a_step(L, ps, L.FP32_DEV, k, None, 96) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
+    assert auto < 1.08 * asked, (auto, asked)
