@@ -48,6 +48,18 @@ int main() {
         const int K = lbh::bounded_nodes(c.b, m, sms);
         CHECK(K == c.K, "D1Q%d, %d members of %d to %d nodes: %d nodes a thread", c.b, c.count, c.lo, c.hi, K);
     }
+    // FP64 windows of a chosen size, or one CTA a member and windows of the default size: what measured
+    // least (both sides over 3% apart)
+    const struct {
+        int b, count, N;
+        bool windows;
+    } w64[] = {{7, 114, 581, false}, {7, 128, 643, false}, {7, 283, 340, false}, {7, 537, 341, false}, {5, 298, 1547, false}, {7, 21, 18787, false},
+               {5, 100, 2048, true}, {7, 1, 300001, true}, {5, 1, 300001, true}, {7, 166, 1000, true}, {5, 80, 2406, true}};
+    for (const auto &c : w64) {
+        int threads = 0, T = 0;
+        const bool got = lbh::windows_f64(c.b, c.b, 4, members(c.count, c.N, c.b), sms, &threads, &T);
+        CHECK(got == c.windows, "D1Q%d, %d members of %d nodes: windows %d", c.b, c.count, c.N, got);
+    }
     if (!fails) std::printf("ok\n");
     return fails ? 1 : 0;
 }

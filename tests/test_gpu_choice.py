@@ -94,3 +94,11 @@ def test_fp32_members_about_a_wave(L, name):
     ps = [periodic(*m) for m in STRIPS[name]]
     auto, asked = (us_a_step(L, ps, L.FP32_DEV, k, None, 96) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
     assert auto < 1.08 * asked, (auto, asked)
+
+
+@pytest.mark.parametrize("eq,count,N", [("kawahara", 114, 581), ("kawahara", 283, 340), ("kawahara", 21, 18787), ("kdv", 298, 1547), ("mkdv", 261, 843)])
+def test_fp64_residents(L, eq, count, N):
+    """FP64 members that fit one CTA each, or windows of the default size, well: they keep them."""
+    ps = [periodic(eq, N)] * count
+    auto, asked = (us_a_step(L, ps, L.FP64, k, None) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
+    assert auto < 1.03 * asked, (auto, asked)
