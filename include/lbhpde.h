@@ -234,7 +234,8 @@ int lbhpde_set_kernel(lbhpde_t h, int kernel, int nodes_per_thread, int steps_pe
  * candidates for one precision, lattice (5 or 7) and f^eq degree on a synthetic periodic grid
  * of 2^22 (FP32) or 2^21 (FP64) nodes in temporally blocked windows, and keeps the fastest in a
  * process-wide table.  Batches and handles created afterwards use the tuned pair in the windows of
- * the on-chip kernel wherever lbhpde_set_kernel did not fix one.  Outputs (each may be NULL): the chosen pair and its
+ * the on-chip kernel wherever lbhpde_set_kernel did not fix one and no other kernel (FP64: no other
+ * size of windows) is estimated to be faster.  Outputs (each may be NULL): the chosen pair and its
  * measured node-updates per second.  Allocates and frees about 235 MB of device memory on the
  * current device and synchronises. */
 int lbhpde_autotune(int precision, int lattice, int degree, int *nodes_per_thread, int *steps_per_launch,

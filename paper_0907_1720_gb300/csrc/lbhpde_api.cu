@@ -496,8 +496,10 @@ int pack_ring(int b, size_t esz, int K, int dc, const std::vector<Member> &m, Pa
 // step: Kawahara on 2000003 nodes, P = 896 and T = 2: 214 (214), P = 768 and T = 4: 216 (216), against 237
 // for P = 1024 and T = 16; 300001 nodes: 33.0 (33) against 47.8; the ensemble of 256 members, P = 384 and
 // T = 4: 70.4 (70.9) against 82.7 with members up to 2048 nodes resident.
-bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps) {
-    const int W = lbk::wmax(b), most = std::min(onchip_maxt_halo(8, b, K), 256) * K, cap = onchip_maxt(8, b, K) * K;
+bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps, int K0, int T0) {
+    if (K0 == 0) K0 = K;
+    const int W = lbk::wmax(b), most = std::min(onchip_maxt_halo(8, b, K), 256) * K, cap = onchip_maxt(8, b, K0) * K0;
+    if (T0 == 0) T0 = default_tblk(cap, W);
     int D = dc > 0 ? dc : 0;
     for (const lbk::Seg &s : m) D = std::max(D, s.D);
     const double us = ((b - 1) * (D + 3) + 1) / 2.0 * 1.039 / 2070.0;  // of one position on an SM
@@ -511,11 +513,11 @@ bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, 
     // a member's last window, which may hold few, starts where it falls and saves nothing) and 0.4 us:
     // 114 D1Q7 members of 581 nodes 11.7 us a step (11.9 predicted), 537 of 341 24.0 (25.9), 21 of 18787 48.0
     // (48.8), D1Q5 253 of 1016 17.5 (17.4), 298 of 1547 28.7 (28.4).
-    const int T0 = default_tblk(cap, W), valid = cap - 2 * T0 * W;
+    const int valid = cap - 2 * T0 * W;
     std::vector<double> ctas;
     auto add = [&](long long warps) {
         const double q = warps / 4.0;
-        ctas.push_back((warps + (warps < 8 ? 0.8 * (std::ceil(q) - q) : 0.0)) * 32 * K * us + 0.4);
+        ctas.push_back((warps + (warps < 8 ? 0.8 * (std::ceil(q) - q) : 0.0)) * 32 * K0 * us + 0.4);
     };
     std::vector<Member> res;
     bool windows = false;
@@ -525,10 +527,10 @@ bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, 
             continue;
         }
         windows = true;
-        for (long long x = 0; x < s.N; x += valid) add(cap / (32 * K));
+        for (long long x = 0; x < s.N; x += valid) add(cap / (32 * K0));
     }
     Packed p;
-    if (!res.empty() && pack_ring(b, 8, K, dc, res, p, cap / K) != LBHPDE_OK) return false;
+    if (!res.empty() && pack_ring(b, 8, K0, dc, res, p, cap / K0) != LBHPDE_OK) return false;
     for (int c = 0; c < p.ncta(); ++c) {
         long long warps = 0;
         for (int i = p.first[c]; i < p.first[c + 1]; ++i) warps += (p.insts[i].nthr + 31) / 32;
@@ -1343,13 +1345,15 @@ int choose_kernels(lbhpde_batch_s *bt) {
         // (3.88e9 node-updates/s against 3.62e9 in windows on a 2^24-node gKdV grid)
         if (g.has_nu && bt->esz == 8 && bt->kernel == LBHPDE_KERNEL_AUTO) continue;
         // FP64: windows of the size and depth that load the SMs evenly, for members of any length
-        // where that beats keeping the short ones resident
+        // where that beats keeping the short ones resident and the tuned or default pair (the autotuner's
+        // depths start at 16 and its grid fills the GPU many times over: D1Q7 on 300001 nodes 47.8 us a step
+        // by its pair, 32.9 so)
         int wthr = 0, wsteps = 0;
-        if (bt->esz == 8 && !g.has_nu && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0 && tk == 0 && sms > 0) {
+        if (bt->esz == 8 && !g.has_nu && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0 && sms > 0) {
             std::vector<Seg> m;
             for (int i : g.members) m.push_back(bt->segs_h[i]);
             const int Kd = lbh::default_K(bt->esz, g.b);
-            if (lbh::windows_f64(g.b, dcg, Kd, m, sms, &wthr, &wsteps)) {
+            if (lbh::windows_f64(g.b, dcg, Kd, m, sms, &wthr, &wsteps, tk, tt)) {
                 K = Kd;
                 tblk = wsteps;
             }

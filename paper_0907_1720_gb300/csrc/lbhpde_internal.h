@@ -110,8 +110,9 @@ void split_ring_classes(size_t esz, int b, int K, const std::vector<Member> &m, 
 int pack_halo(int b, size_t esz, int K, int dc, int H, const std::vector<Member> &m, Packed &out,
               bool wide = false, int threads = 0);
 // Whether FP64 periodic members advance faster in windows of a chosen size alone (threads of a CTA,
-// steps a launch) than with the short ones resident and the long ones in windows of the default size.
-bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps);
+// steps a launch) than with the short ones resident and the long ones in windows of a CTA's size, with K0
+// nodes a thread and T0 steps a launch (0: K and the default).
+bool windows_f64(int b, int dc, int K, const std::vector<lbk::Seg> &m, int sms, int *threads, int *steps, int K0 = 0, int T0 = 0);
 
 // K == kRingK launches k_ring (resident plans only).
 int launch_onchip(int b, size_t esz, int K, int dc, bool halo, const Packed &p, const lbk::OnchipInst *insts_d,

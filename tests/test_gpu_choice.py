@@ -102,3 +102,16 @@ def test_fp64_residents(L, eq, count, N):
     ps = [periodic(eq, N)] * count
     auto, asked = (us_a_step(L, ps, L.FP64, k, None) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
     assert auto < 1.03 * asked, (auto, asked)
+
+
+@pytest.mark.parametrize("eq,b,N", [("kawahara", 7, 300001), ("kdv", 5, 300001)])
+def test_tuning_is_not_slower(L, eq, b, N):
+    """An FP64 grid after the autotuner has recorded its pair against the same grid before."""
+    ps = [periodic(eq, N)]
+    before = us_a_step(L, ps, L.FP64, L.KERNEL_AUTO, None)
+    try:
+        L.autotune(L.FP64, b, b)
+        after = us_a_step(L, ps, L.FP64, L.KERNEL_AUTO, None)
+    finally:
+        L.set_tuning(L.FP64, b, b, 4, 64 if b == 5 else 16)  # the untuned pair
+    assert after < 1.05 * before, (after, before)
