@@ -387,11 +387,14 @@ int plan_block(lbhpde_server_s *S, Block &blk) {
     // FP32 windows of 128 threads (1024 nodes, 32 steps a launch) while the requests in flight leave
     // SMs idle, of a resident CTA's size otherwise, when the wider ones' smaller share of copies counts
     // (GB300, ms a burst, wide and narrow: 8 requests 8.0 and 5.0, 12 5.2 and 3.1, 24 with 279 000 nodes
-    // 9.6 and 6.3; 48 with 558 000 nodes 13.7 and 14.6, 200 29.9 and 32.4)
-    long long in_flight = 0;
+    // 9.6 and 6.3; 48 with 558 000 nodes 13.7 and 14.6, 200 29.9 and 32.4).  A D1Q7 node counts two and a half:
+    // narrow windows of 4 nodes a thread are 512 positions there, 192 of them copies (2048 steps: D1Q5 200 000
+    // nodes 2.39 and 1.91; D1Q7 100 003 2.17 and 2.14, 160 000 3.06 and 3.14, 200 000 2.40 and 2.93; of both half
+    // 160 000 2.57 and 2.34, 288 000 3.21 and 3.87)
+    long long in_flight = 0;  // half nodes of D1Q5
     for (const Req *r : S->active)
-        if (r->done < r->nsteps) in_flight += r->N;
-    const bool narrow = S->esz == 4 && in_flight < 2000LL * S->sms;
+        if (r->done < r->nsteps) in_flight += (r->mi.b == 5 ? 2 : 5) * r->N;
+    const bool narrow = S->esz == 4 && in_flight < 4000LL * S->sms;
     // per lattice, three classes: requests whose f^eq degree the compiled variant covers (D <= 5
     // on D1Q5, <= 7 on D1Q7), higher-degree polynomials, and real-exponent models, each with its
     // own launches, so that one high-degree or real-exponent request does not send the whole

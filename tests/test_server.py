@@ -265,3 +265,17 @@ def test_divergent_request_is_reported(L):
     rc, phi, info = srv.wait(ok, timeout=60)
     assert rc == L.OK and info["nonfinite"] == 0
     srv.close()
+
+
+@pytest.mark.parametrize("eq,dt,N,launches", [("kdv", 1e-4, 200003, 32), ("kawahara", 1e-3, 200003, 16), ("kawahara", 1e-3, 50021, 32)])
+def test_fp32_window_size_by_lattice(L, eq, dt, N, launches):
+    """A long request takes narrow windows (32 steps a launch) while the nodes in flight leave SMs idle,
+    wide ones (64) otherwise; a D1Q7 node's narrow windows fill them two and a half times as much."""
+    srv = L.Server(precision=L.FP32_DEV, device_bytes=64 << 20, max_active=8, steps_per_block=256)
+    p = W.Problem(getattr(W, eq)(), N, 0.1, dt, 2.5 if eq == "kawahara" else 1.3, 1024, bump(N, 0.1, 3))
+    st, phi, _ = srv.wait(srv.submit_problem(p))
+    n = srv.stats()["launches"]
+    srv.close()
+    s = L.Solver.for_problem(p, precision=L.FP32_DEV).set_phi(p.phi0).step(1024)
+    assert st == L.OK and np.array_equal(phi, s.read_phi()) and n == launches
+    s.close()
