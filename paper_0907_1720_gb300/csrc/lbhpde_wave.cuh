@@ -558,8 +558,7 @@ __global__ void __launch_bounds__(32 * kWaveWarps)
         cluster_sync();  // no CTA ends while a neighbour may still write into its boxes
     } else if (used) {
         // the last window to finish moves the trades' numbers on for the next launch, after every
-        // window has read them
-        fence();
+        // window has read them (they all have before their fence above)
         if (lane == 0 && atomicAdd(ctrl + 1, 1u) == (unsigned)(nused - 1)) {
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
             ctrl[1] = 0;
