@@ -89,7 +89,7 @@ struct Group {
     int *smembers = nullptr;
     std::vector<int2> sblocks_h;       // their node blocks (kChunk nodes each)
     int2 *sblocks = nullptr;
-    // the whole batch in one-warp windows (then the plans above are empty)
+    // the whole batch in one-warp windows (then the plans above serve calls of few steps, if any)
     lbh::PackedWave wv_h;
     lbk::WaveWin *wv_wins = nullptr;
     unsigned char *wv_box = nullptr;
@@ -97,6 +97,7 @@ struct Group {
     int *wv_members = nullptr;  // bounded: the batch indices of the plan's members,
     void *wv_ends = nullptr;    //   and f^eq(phi_b) of the steps of a launch,
     int wv_steps = 0;           //   as many as this holds
+    long wv_few = 0;            // calls of fewer steps take the resident kernels, planned beside the windows
 };
 
 }  // namespace
@@ -1277,6 +1278,16 @@ int plan_waves(lbhpde_batch_s *bt, bool *taken) {
         RC(bt->upload(&g->wv_members, g->members));
         RC(bt->dev_alloc(&g->wv_ends, per * g->wv_steps));
     }
+    // A call of few FP32 steps costs its launches: the trades of a cluster's windows and the ends' own
+    // launch are 0.8 and 4 us more than a resident kernel's one launch, which a step gains back one by one
+    // (GB300, us a call, resident and windows: KdV on 400 nodes 1 step 4.1 and 5.2, 8 steps 6.2 and 6.2;
+    // Example 4.5 on 601 nodes 1 step 6.2 and 10.3, 4 8.3 and 10.3, 16 20.5 and 14.4).  In place like the
+    // windows, and with the same bits.
+    const bool fits = std::all_of(g->members.begin(), g->members.end(), [&](int i) {
+        return bt->N[i] <= (nee ? (long long)lbh::kBoundedK * lbh::kBoundedMaxT : (long long)lbh::onchip_maxt(bt->esz, g->b, 8) * 8);
+    });
+    g->wv_few = 0;
+    if (bt->esz == 4 && fits) g->wv_few = (long)std::ceil((nee ? 4.0 : 0.8) * 2070 / std::max(1.0, g->wv_h.other - g->wv_h.cost));
     *taken = true;
     return LBHPDE_OK;
 }
@@ -1292,11 +1303,11 @@ int choose_kernels(lbhpde_batch_s *bt) {
     }
     bool taken = false;
     RC(plan_waves(bt, &taken));
-    if (taken) return LBHPDE_OK;
     for (auto &g : bt->groups) {
         if (g.members.empty()) continue;
         g.onchip_ok = false;
         drop_strip(bt, g);
+        if (taken && g.wv_few <= 1) continue;
         if (bt->kernel == LBHPDE_KERNEL_STREAM) continue;
         // K_req = kRingK asks for the 16-node resident kernel, whose windows keep the default (or
         // tuned) K; automatic choice: that kernel wherever it applies
@@ -1316,12 +1327,12 @@ int choose_kernels(lbhpde_batch_s *bt) {
             sms = 0;
         }
         // strips wherever they are the faster kernel (lbh::strip_cost against lbh::cta_cost)
-        if (bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0) {
+        if (!taken && bt->kernel == LBHPDE_KERNEL_AUTO && bt->K_req == 0 && bt->spl_req == 0) {
             bool done = false;
             RC(plan_strip(bt, g, sms, &done));
             if (done) continue;
         }
-        const bool small = bt->K_req == 0 && bt->kernel != LBHPDE_KERNEL_HALO && thr16 < 32LL * sms;
+        const bool small = bt->K_req == 0 && bt->kernel != LBHPDE_KERNEL_HALO && (taken || thr16 < 32LL * sms);
         int K_small = 0;
         if (small)
             for (int Kc : {2, 4, 8})
@@ -1361,8 +1372,11 @@ int choose_kernels(lbhpde_batch_s *bt) {
         int rc = plan_onchip(bt, g, K, ring16 ? lbh::kRingK : K, tblk, bt->kernel == LBHPDE_KERNEL_HALO || wthr > 0, wthr);
         if (rc != LBHPDE_OK) return rc;
     }
-    for (auto &g : bt->bgroups)
-        if (!g.members.empty()) RC(plan_bounded(bt, g));
+    for (auto &g : bt->bgroups) {
+        if (g.members.empty() || (taken && g.wv_few <= 1)) continue;
+        RC(plan_bounded(bt, g));
+        if (!g.smembers_h.empty()) g.wv_few = 0;  // (streamed: through both buffers)
+    }
     return LBHPDE_OK;
 }
 
@@ -1657,7 +1671,7 @@ int batch_step(lbhpde_batch_s *bt, long nsteps, const double *phib = nullptr, lo
     if (bt->nbounded) RC(stage_boundary(bt, nsteps, phib, stride, on_device, &pbd));
     for (int gi = 0; gi < 4; ++gi) {
         Group &g = gi < 2 ? bt->groups[gi] : bt->bgroups[gi - 2];
-        if (g.wv_h.wins.empty()) continue;
+        if (g.wv_h.wins.empty() || nsteps < g.wv_few) continue;
         for (long done = 0; done < nsteps;) {  // the whole batch, in place
             const int n = (int)std::min<long>(nsteps - done, bt->nbounded ? g.wv_steps : 1L << 30);
             if (bt->nbounded) {

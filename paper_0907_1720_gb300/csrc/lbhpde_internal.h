@@ -187,6 +187,7 @@ struct PackedWave {
     int tblk = 0;      // steps between two trades of the windows' borders
     int csize = 0;     // CTAs of a cluster that holds whole instances; 0: boxes in global memory
     int nmem = 0, nused = 0;  // members; windows that hold nodes
+    double cost = 0, other = 0;  // modelled clocks of a step, and of a step of the best other kernel
     int wsmem = 0;     // shared-memory elements a window, beside the boxes
     size_t smem = 0, box_bytes = 0;
     int ncta() const { return (int)wins.size() / lbk::kWaveWarps; }

@@ -446,6 +446,8 @@ bool plan_wave(size_t esz, int b, int dc, bool nee, const std::vector<lbk::Seg> 
         out.tblk = k.T;
         out.csize = k.C;
         out.nmem = (int)m.size();
+        out.cost = k.cost;
+        out.other = other;
         if (!pack_wave(m, b, k.K, k.G, k.T, k.C, out.wins)) continue;
         out.nused = (int)std::count_if(out.wins.begin(), out.wins.end(), [](const lbk::WaveWin &w) { return w.N > 0; });
         out.wsmem = ((nee ? lbk::wave_end_elems(b, k.T) : 0) + (dc > 0 ? 0 : lbk::wave_coef_elems(b, D)) + 3) & ~3;

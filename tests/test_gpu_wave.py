@@ -164,3 +164,39 @@ def test_wait_that_runs_out(L, tmp_path):
     assert r.returncode == 0, r.stderr[-2000:]
     out = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert out.returncode == 0 and out.stdout.startswith("ok"), out.stdout[-2000:]
+
+
+@pytest.mark.parametrize("example,N,depth", [("4.1", 96, 2), ("4.1", 601, 2), ("4.1", 1024, 2), ("4.5", 129, 2), ("4.5", 601, 1), ("4.5", 768, 2)])
+def test_bounded_fp32_member_alone_and_in_a_batch(L, example, N, depth):
+    """FP32 members that a large batch gives a warp each: the one-warp windows alone (two launches a
+    call: the ends' values and the steps; one where a few steps go to the resident kernel), equal to
+    the streaming step and to the same member among many."""
+    p = bounded(example, N, depth)
+    pb = W.boundary_values(p, 2 if example == "4.1" else 3, 0, 60)
+    want, _ = solve(L, [p], 1, L.KERNEL_STREAM, [1, 2, 57], pb)
+    alone, n = solve(L, [p], 1, L.KERNEL_AUTO, [1, 2, 57], pb)
+    one, n1 = solve(L, [p], 1, L.KERNEL_AUTO, [57, 2, 1], pb)
+    many, nm = solve(L, [p] * 700, 1, L.KERNEL_AUTO, [1, 2, 57], pb)
+    assert n == 2 and n1 == 1 and nm == 1
+    assert np.isfinite(want).all() and np.array_equal(alone, want) and np.array_equal(one, want)
+    assert np.array_equal(many.reshape(700, N), np.broadcast_to(want, (700, N)))
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("eq", list(EQS) + ["gks_cubic"])
+@pytest.mark.parametrize("N", [33, 400, 1537])
+def test_periodic_few_steps_and_many(L, eq, N, prec):
+    """Calls of a few steps (resident in FP32) and of many (windows) on one state, one launch each; also
+    a run-time degree (gks_cubic: 13)."""
+    if eq == "gks_cubic":
+        phi0 = 0.4 + 0.3 * np.cos(2 * np.pi * np.arange(N) / N)
+        p = W.Problem(W.gks_cubic(), N, 0.1, 1e-5, 1.2, 0, phi0)
+    else:
+        p = problem(eq, N, 0)
+    calls = [1, 40, 2, 3, 33, 1, 1]
+    b, _ = solve(L, [p], prec, L.KERNEL_STREAM, [sum(calls)])
+    for c in (calls, calls + [64]):
+        a, n = solve(L, [p], prec, L.KERNEL_AUTO, c)
+        assert n == 1
+        if c is calls:
+            assert np.isfinite(b).all() and np.array_equal(a, b)
