@@ -110,7 +110,7 @@ struct lbhpde_batch_s {
     // launches of disjoint members run on `side`, forked from and joined back into `stream` with
     // events, so that one fills the SMs another leaves idle
     cudaStream_t side[kSides] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
+    cudaEvent_t ev_fork = nullptr, ev_started = nullptr, ev_join[kSides] = {};
     // side stream i, waiting for what `stream` held at the fork (ev_fork has been recorded)
     int fork_side(int i, cudaStream_t *st) {
         if (!side[i]) {
@@ -224,7 +224,8 @@ struct lbhpde_batch_s {
             ev_join[c] = nullptr;
         }
         if (ev_fork) cudaEventDestroy(ev_fork);
-        ev_fork = nullptr;
+        if (ev_started) cudaEventDestroy(ev_started);
+        ev_fork = ev_started = nullptr;
         stream = nullptr;
     }
 };
@@ -1604,16 +1605,28 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
         // 1459 nodes 50, 140 and 79, 359; 6 of 327 to 1309 20, 65 and 41, 211)
         const bool fork = kinds.size() > 1;
         if (fork) RC(bt->record_fork());
+        // A CTA of k_ring_nee takes a whole SM: the others wait until its CTAs are placed, else a warp of
+        // theirs on each SM could hold them all off (where the stream has work before the fork, both are
+        // ready at once).  Not in a capture, where the launches' order has to do.
+        cudaEvent_t started = nullptr;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (fork && kinds[0].what == kRingNee && (bt->stream == nullptr || cudaStreamIsCapturing(bt->stream, &cap) == cudaSuccess) &&
+            cap == cudaStreamCaptureStatusNone) {
+            if (!bt->ev_started) CK(cudaEventCreateWithFlags(&bt->ev_started, cudaEventDisableTiming));
+            started = bt->ev_started;
+        }
         bool used[kSides] = {};
         auto launch = [&](size_t i) -> int {
             Group &g = *kinds[i].g;
             cudaStream_t st = bt->stream;
             const int sd = (int)((i + kSides - 1) % kSides);  // (the first on the batch's own stream)
             if (fork && i > 0) {
-                if (used[sd])
+                if (used[sd]) {
                     st = bt->side[sd];
-                else
+                } else {
                     RC(bt->fork_side(sd, &st));
+                    if (started) CK(cudaStreamWaitEvent(st, started, 0));
+                }
                 used[sd] = true;
             }
             for (long done = 0; done < nsteps;) {
@@ -1622,7 +1635,8 @@ int step_bounded(lbhpde_batch_s *bt, long nsteps, const double *pbd, long long s
                 int n;
                 if (kinds[i].what == kRingNee) {
                     n = (int)std::min<long>(nsteps - done, 1L << 30);
-                    RC(lbh::launch_ring_nee_f32(g.rn_dc, g.rn_h, g.rn_insts, g.rn_first, in, out, bt->coefT, pbd, stride, done, n, st));
+                    RC(lbh::launch_ring_nee_f32(g.rn_dc, g.rn_h, g.rn_insts, g.rn_first, in, out, bt->coefT, pbd, stride, done, n, st,
+                                                i == 0 && done == 0 ? started : nullptr));
                 } else if (kinds[i].what == kSpan) {
                     n = (int)std::min<long>(nsteps - done, 1L << 28);
                     RC(lbh::launch_span(g.b, kinds[i].K, g.sp + kinds[i].first, kinds[i].count, in, out,

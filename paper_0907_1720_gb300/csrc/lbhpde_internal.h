@@ -174,9 +174,10 @@ struct NeeMember {
 // 512-thread CTA, depth within the first and last 16 interior nodes' reach.
 bool ring_nee_ok(size_t esz, int b, const lbk::Seg &s);
 int pack_ring_nee(int b, int dc, const std::vector<NeeMember> &m, PackedNee &out, int threads);
+// started: an event to record once every CTA has begun (best effort; nullptr: none).
 int launch_ring_nee_f32(int dc, const PackedNee &p, const lbk::RingNeeInst *insts_d, const int *first_d,
                         const void *in, void *out, const void *coefT, const double *phib, long long stride,
-                        long long step0, int nsteps, cudaStream_t st);
+                        long long step0, int nsteps, cudaStream_t st, cudaEvent_t started = nullptr);
 
 // Small and medium grids in windows of one warp each (k_wave, lbhpde_wave.cu).
 struct PackedWave {

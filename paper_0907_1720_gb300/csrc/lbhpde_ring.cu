@@ -50,25 +50,40 @@ namespace {
 template <int MAXT, int DC, bool D2>
 int launch_ring_nee_t(const PackedNee &p, const lbk::RingNeeInst *insts, const int *first, const void *in, void *out,
                       const void *coefT, const double *phib, long long stride, long long step0, int nsteps,
-                      cudaStream_t st) {
+                      cudaStream_t st, cudaEvent_t started) {
     auto fn = lbk::k_ring_nee<float, 5, kRingK, MAXT, DC, D2>;
     if (!allow_smem(fn)) return LBHPDE_ERR_CUDA;
-    fn<<<p.ncta(), p.nthreads, p.smem, st>>>((const float *)in, (float *)out, insts, first, (const float *)coefT, phib,
-                                             stride, step0, nsteps);
-    if (cudaGetLastError() != cudaSuccess) return LBHPDE_ERR_CUDA;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)p.ncta());
+    cfg.blockDim = dim3((unsigned)p.nthreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    if (started) {  // recorded once every CTA has begun
+        at[0].id = cudaLaunchAttributeLaunchCompletionEvent;
+        at[0].val.launchCompletionEvent.event = started;
+        at[0].val.launchCompletionEvent.flags = 0;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+    if (cudaLaunchKernelEx(&cfg, fn, (const float *)in, (float *)out, insts, first, (const float *)coefT, phib, stride, step0, nsteps) !=
+        cudaSuccess) {
+        (void)cudaGetLastError();
+        return LBHPDE_ERR_CUDA;
+    }
     return LBHPDE_OK;
 }
 
 template <int MAXT>
 int launch_ring_nee_d(int dc, const PackedNee &p, const lbk::RingNeeInst *insts, const int *first, const void *in,
                       void *out, const void *coefT, const double *phib, long long stride, long long step0, int nsteps,
-                      cudaStream_t st) {
+                      cudaStream_t st, cudaEvent_t started) {
     if (dc == 5 && p.d2)
-        return launch_ring_nee_t<MAXT, 5, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
-    if (dc == 5) return launch_ring_nee_t<MAXT, 5, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
+        return launch_ring_nee_t<MAXT, 5, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st, started);
+    if (dc == 5) return launch_ring_nee_t<MAXT, 5, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st, started);
     if (dc >= 0 && p.d2)
-        return launch_ring_nee_t<MAXT, 0, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
-    if (dc >= 0) return launch_ring_nee_t<MAXT, 0, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st);
+        return launch_ring_nee_t<MAXT, 0, true>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st, started);
+    if (dc >= 0) return launch_ring_nee_t<MAXT, 0, false>(p, insts, first, in, out, coefT, phib, stride, step0, nsteps, st, started);
     return LBHPDE_ERR_UNSUPPORTED;
 }
 
@@ -152,13 +167,13 @@ int pack_ring_nee(int b, int dc, const std::vector<NeeMember> &m, PackedNee &out
 
 int launch_ring_nee_f32(int dc, const PackedNee &p, const lbk::RingNeeInst *insts_d, const int *first_d,
                         const void *in, void *out, const void *coefT, const double *phib, long long stride,
-                        long long step0, int nsteps, cudaStream_t st) {
+                        long long step0, int nsteps, cudaStream_t st, cudaEvent_t started) {
     if (p.ncta() == 0 || nsteps <= 0) return LBHPDE_OK;
     if (p.nthreads > p.stride || p.nthreads % 32 != 0) return LBHPDE_ERR_ARG;
     for (int c = 0; c < p.ncta(); ++c)  // every helper role has its thread
         if ((p.first[c + 1] - p.first[c]) * lbk::nee_roles(5) > p.nthreads) return LBHPDE_ERR_ARG;
     if (p.stride == 512)
-        return launch_ring_nee_d<512>(dc, p, insts_d, first_d, in, out, coefT, phib, stride, step0, nsteps, st);
+        return launch_ring_nee_d<512>(dc, p, insts_d, first_d, in, out, coefT, phib, stride, step0, nsteps, st, started);
     return LBHPDE_ERR_UNSUPPORTED;
 }
 

@@ -115,3 +115,12 @@ def test_tuning_is_not_slower(L, eq, b, N):
     finally:
         L.set_tuning(L.FP64, b, b, 4, 64 if b == 5 else 16)  # the untuned pair
     assert after < 1.05 * before, (after, before)
+
+
+@pytest.mark.parametrize("count,lo,hi", [(2444, 64, 102), (226, 280, 1123)])
+def test_bounded_beside_a_periodic_member(L, count, lo, hi):
+    """FP32 bounded members on both of their kernels, behind a periodic member's launch on the stream."""
+    ps = [periodic("kdv", 64)] + [bounded("ks", N) for N in spread(count, lo, hi)]
+    phib = torch.from_numpy(W.boundary_values(ps[1], 2, 0, 48)).cuda()
+    auto, asked = (us_a_step(L, ps, L.FP32_DEV, k, phib) for k in (L.KERNEL_AUTO, L.KERNEL_ONCHIP))
+    assert auto < 1.06 * asked, (auto, asked)
