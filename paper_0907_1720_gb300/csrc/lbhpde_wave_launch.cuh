@@ -261,7 +261,7 @@ namespace {
 // warp takes the writes past its members' ends once for each remainder of 16 [1318 members of 43 to 173
 // nodes 3930, 431 of 133 to 534 2600, 303 of 455 to 1821 2080; equal members of any size 1600 to 1700].
 double ring_cost(const std::vector<lbk::Seg> &m, int sms) {
-    std::vector<Member> res, full, tail, cls[kRingClasses];
+    std::vector<Member> res, cls[kRingClasses];
     long long nodes = 0;
     bool equal = true;
     for (const lbk::Seg &s : m)
@@ -271,10 +271,8 @@ double ring_cost(const std::vector<lbk::Seg> &m, int sms) {
             equal = equal && s.N % kRingK == res[0].seg.N % kRingK;
         }
     if (res.empty()) return 0;
-    if (split_ring_waves(5, kRingK, sms, res, full, tail)) {
-        const double waves = nodes / (512.0 * kRingK * sms), rest = waves - std::floor(waves);
-        return 3400 * (std::floor(waves) + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0)));
-    }
+    const double waves = nodes / (512.0 * kRingK * sms), rest = waves - std::floor(waves);
+    if (waves >= 1) return 3400 * (std::floor(waves) + (rest > 0.25 ? 1.0 : (rest > 0 ? 0.6 : 0.0)));
     split_ring_classes(4, 5, kRingK, res, cls);
     std::vector<int> load(sms, 0);  // warps, the largest CTAs first, each to the emptiest SM (a heap)
     for (int c = kRingClasses - 1; c >= 0; --c) {
