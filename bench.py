@@ -259,6 +259,12 @@ def gather_member_records(records, world, device="cpu"):
     return sorted((int(r[0]), r[1], r[2], int(r[3])) for r in out)
 
 
+def chosen_kernel(name, fills):
+    """The kernel's name where the members surely take it (they fill the GPU); elsewhere what the automatic
+    choice takes them from, by their sizes and number."""
+    return name if fills else f"the automatic choice among k_wave, k_strip, k_ring, k_onchip, k_span and k_bounded (filled GPU: {name})"
+
+
 def run_ours(args, rank, world, cpu=None):
     import torch
 
@@ -397,8 +403,9 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": ("k_span<5,20> (one warp per instance, its nodes in registers)" if esz == 4 else
-                               "k_bounded<double,5,K,512,5> (one resident CTA per instance, 3 to 6 nodes a thread)"),
+                    "kernel": chosen_kernel("k_span<5,20> (one warp per instance, its nodes in registers)" if esz == 4 else
+                                            "k_bounded<double,5,K,MAXT,5> (one resident CTA per instance, 3 to 6 nodes a thread)",
+                                            len(probs) >= 2 * sms and probs[0].N == 601),
                     "flops_per_node_update": fl, "peak_source": src}
         elif args.workload == "nu_grid" and args.kernel != "stream":
             A, Dg = nu_shape(L, probs[0])
@@ -407,8 +414,8 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": ("k_strip<5,9,4,1> (strips of one warp, phi^nu)" if esz == 4 else
-                               "k_stream_rt<double,5,256> (run-time degree, phi^nu)"),
+                    "kernel": chosen_kernel("k_strip<5,9,4,1> (strips of one warp, phi^nu)" if esz == 4 else
+                                            "k_stream_rt<double,5,256> (run-time degree, phi^nu)", total >= 1 << 21),
                     "flops_per_node_update": fl, "peak_source": src}
         elif args.workload == "nu_grid":
             by = bytes_per_node_update(b, esz)
@@ -423,8 +430,8 @@ def run_ours(args, rank, world, cpu=None):
             achieved = fl * upd_step / (kern_ms / 1e3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf, "traffic": None,
-                    "kernel": (f"k_strip<{b},{D}> (strips of one warp, 16 steps a launch)" if esz == 4 else
-                               f"k_onchip<double,{b},K> (windows that load the SMs evenly)"),
+                    "kernel": chosen_kernel(f"k_strip<{b},{D}> (strips of one warp, 16 steps a launch)" if esz == 4 else
+                                            f"k_onchip<double,{b},K> (windows that load the SMs evenly, or by the tuned pair)", total >= 1 << 21),
                     "flops_per_node_update": fl, "peak_source": src}
         else:
             by = bytes_per_node_update(b, esz)

@@ -1,8 +1,8 @@
 // Bounded FP32 instances of up to 1024 nodes (D1Q5, depth 2) or 768 (D1Q7, depth 1 or 2), one warp each
 // for every step of a launch (the boundary rule of lbhpde_bounded.cuh).
 //
-// A lane holds K nodes in registers (node x at lane x / K, register x % K; K = 4 to 32, the smallest
-// multiple of 4 that holds the instance; 8 to 24 on D1Q7), its neighbours' edges come by shuffle, and nothing is
+// A lane holds K nodes in registers (node x at lane x / K, register x % K; K = 4 to 32, at least the
+// smallest multiple of 4 that holds the instance; 8 to 24 on D1Q7), its neighbours' edges come by shuffle, and nothing is
 // shared with other warps: no barrier, no exchange buffer, no copies.  The bound is the FP32 pipes
 // (and below 300 nodes the ends, which cost a warp the same at any size); in k_ring_nee, whose
 // 512-thread CTAs hold 13 instances of 601 nodes, every step waits at a barrier, and in k_bounded
