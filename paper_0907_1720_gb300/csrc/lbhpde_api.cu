@@ -1371,12 +1371,18 @@ int choose_kernels(lbhpde_batch_s *bt) {
             }
         }
         int rc = plan_onchip(bt, g, K, ring16 ? lbh::kRingK : K, tblk, bt->kernel == LBHPDE_KERNEL_HALO || wthr > 0, wthr);
-        if (rc != LBHPDE_OK) return rc;
+        if (taken && rc != LBHPDE_OK)
+            g.wv_few = 0;  // the windows take every call
+        else
+            RC(rc);
     }
     for (auto &g : bt->bgroups) {
         if (g.members.empty() || (taken && g.wv_few <= 1)) continue;
-        RC(plan_bounded(bt, g));
-        if (!g.smembers_h.empty()) g.wv_few = 0;  // (streamed: through both buffers)
+        const int rc = plan_bounded(bt, g);
+        if (taken && (rc != LBHPDE_OK || !g.smembers_h.empty()))
+            g.wv_few = 0;  // (streamed members go through both buffers)
+        else
+            RC(rc);
     }
     return LBHPDE_OK;
 }
